@@ -612,6 +612,7 @@ __global__ void __launch_bounds__(256) k_jac_sell_rz(const int *__restrict__ row
   const bool valid = i < tl.row1[t];
   pdl_wait();
   pdl_trigger();
+  if (ks[sys].done) return;   // uniform in the block: one system per tile
   double rz = 0.0;
   if (valid) {
     T zi;
@@ -623,11 +624,10 @@ __global__ void __launch_bounds__(256) k_jac_sell_rz(const int *__restrict__ row
     }
     rz = (double)fma(r[i], zi, (T)0);
   }
-  if (ks[sys].done) return;   // uniform in the block: one system per tile
   double v[1] = {rz}, out[1];
   if (seg_sum<256, 1>(v, partials, counter, tl, t, sys, out) && threadIdx.x == 0) {
     KrylovScalars &k = ks[sys];
-    k.beta = out[0] / k.rz;
+    k.beta = k.rz > 0.0 ? out[0] / k.rz : 0.0;   // 0 in the first iteration (rz starts at 0)
     k.rz = out[0];
     if (!(out[0] > 0.0)) { k.breakdown = 1; k.done = 1; atomicAdd(n_done, 1); }
   }

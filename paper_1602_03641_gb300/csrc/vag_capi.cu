@@ -182,13 +182,9 @@ void destroy_system(vag_system *sys) {
   System *s = &sys->s;
   Ctx *c = s->ctx;
   if (c && c->stream) cudaStreamSynchronize(c->stream);
-  if (s->pcg_graph) cudaGraphExecDestroy(s->pcg_graph);
-  if (s->mx.graph) cudaGraphExecDestroy(s->mx.graph);
-  if (s->mx.graph_amg) cudaGraphExecDestroy(s->mx.graph_amg);
-  if (s->pcg_graph_amg) cudaGraphExecDestroy(s->pcg_graph_amg);
+  for (LoopGraph *g : {&s->pcg_loop, &s->pcg_loop_amg, &s->pcg_loop_cheb, &s->bicg_loop, &s->mx.loop, &s->mx.loop_amg})
+    loop_destroy(*g);
   if (s->step_graph) cudaGraphExecDestroy(s->step_graph);
-  if (s->bicg_graph) cudaGraphExecDestroy(s->bicg_graph);
-  if (s->pcg_graph_cheb) cudaGraphExecDestroy(s->pcg_graph_cheb);
   amg_free(s);
   if (s->ks_host) cudaFreeHost(s->ks_host);
   if (s->n_done_host) cudaFreeHost(s->n_done_host);

@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(NT) k_cheb_step(const int *__restrict__ rowptr
   double v[1] = {rz}, out[1];
   if (seg_sum<NT, 1>(v, partials, counter, tl, t, sys, out) && threadIdx.x == 0) {
     KrylovScalars &k = ks[sys];
-    k.beta = out[0] / k.rz;
+    k.beta = k.rz > 0.0 ? out[0] / k.rz : 0.0;   // 0 in the first iteration (rz starts at 0)
     k.rz = out[0];
     if (!(out[0] > 0.0)) { k.breakdown = 1; k.done = 1; atomicAdd(n_done, 1); }
   }

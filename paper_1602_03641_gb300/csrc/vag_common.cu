@@ -60,6 +60,45 @@ void trace_report(const char *call) {
   t_marks.clear();
 }
 
+void loop_destroy(LoopGraph &g) {
+  if (g.exec) cudaGraphExecDestroy(g.exec);
+  g = LoopGraph{};
+}
+
+void loop_build(LoopGraph &g, cudaStream_t st, const std::function<void(cudaGraphConditionalHandle)> &body) {
+  loop_destroy(g);
+  struct Graph {   // released on every path
+    cudaGraph_t g = nullptr;
+    ~Graph() {
+      if (g) cudaGraphDestroy(g);
+    }
+  } top;
+  VAG_CUDA(cudaGraphCreate(&top.g, 0));
+  cudaGraphConditionalHandle h;
+  VAG_CUDA(cudaGraphConditionalHandleCreate(&h, top.g, 1, cudaGraphCondAssignDefault));
+  cudaGraphNodeParams p{};
+  p.type = cudaGraphNodeTypeConditional;
+  p.conditional.handle = h;
+  p.conditional.type = cudaGraphCondTypeWhile;
+  p.conditional.size = 1;
+  cudaGraphNode_t node;
+  VAG_CUDA(cudaGraphAddNode(&node, top.g, nullptr, nullptr, 0, &p));
+  cudaGraph_t inner = p.conditional.phGraph_out[0];   // owned by the conditional node
+  VAG_CUDA(cudaStreamBeginCaptureToGraph(st, inner, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
+  set_capturing(true);
+  try {
+    body(h);
+  } catch (...) {
+    set_capturing(false);
+    cudaStreamEndCapture(st, &inner);
+    throw;
+  }
+  set_capturing(false);
+  VAG_CUDA(cudaStreamEndCapture(st, &inner));
+  VAG_CUDA(cudaGraphGetNodes(inner, nullptr, &g.nodes));
+  VAG_CUDA(cudaGraphInstantiate(&g.exec, top.g, 0));
+}
+
 void *ctx_alloc(Ctx *c, size_t bytes) {
   void *p = nullptr;
   cudaError_t e = c->pool ? cudaMallocFromPoolAsync(&p, bytes, c->pool, c->stream) : cudaMalloc(&p, bytes);

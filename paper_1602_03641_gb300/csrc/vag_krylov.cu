@@ -15,8 +15,8 @@
 // A converged system's tiles return at entry.  Reductions are deterministic
 // and depend only on the system itself (its tiles cover its own rows only),
 // so a system gives bitwise the same iterates alone or in a batch.
-// Iterations are captured in a CUDA graph of `chunk` iterations; the host
-// polls one counter (systems done) between graph launches.
+// Iterations run in a CUDA graph loop that the device ends when every system
+// is done (no host poll, and no iteration past the last).
 #include <cmath>
 #include <cstdio>
 #include <vector>
@@ -105,9 +105,11 @@ __global__ void __launch_bounds__(NT) k_update(double *__restrict__ x, double *_
                                                unsigned *counter, KrylovScalars *ks, int *n_done) {
   const int t = blockIdx.x;
   const int sys = tl.sys[t];
+  const int r0 = tl.row0[t], r1 = tl.row1[t];
+  pdl_wait();
+  pdl_trigger();
   if (ks[sys].done) return;
   const double alpha = ks[sys].alpha;
-  const int r0 = tl.row0[t], r1 = tl.row1[t];
   double rz = 0.0, rr = 0.0;
   for (int i = r0 + threadIdx.x; i < r1; i += NT) {
     x[i] = fma(alpha, p[i], x[i]);
@@ -130,12 +132,16 @@ __global__ void __launch_bounds__(NT) k_update(double *__restrict__ x, double *_
 }
 
 __global__ void __launch_bounds__(NT) k_pdir(double *__restrict__ p, const double *__restrict__ r,
-                                             const double *__restrict__ dinv, Tiles tl, const KrylovScalars *ks) {
+                                             const double *__restrict__ dinv, Tiles tl, const KrylovScalars *ks,
+                                             int check, cudaGraphConditionalHandle loop, int *n_done) {
   const int t = blockIdx.x;
   const int sys = tl.sys[t];
+  const int r0 = tl.row0[t], r1 = tl.row1[t];
+  pdl_wait();
+  pdl_trigger();
+  if (check && t == 0 && threadIdx.x == 0) loop_end_check(loop, n_done, tl.n_sys);
   if (ks[sys].done) return;
   const double beta = ks[sys].beta;
-  const int r0 = tl.row0[t], r1 = tl.row1[t];
   for (int i = r0 + threadIdx.x; i < r1; i += NT) p[i] = fma(beta, p[i], dinv[i] * r[i]);
 }
 
@@ -171,10 +177,14 @@ __global__ void __launch_bounds__(NT) k_restart(const double *__restrict__ b, co
 
 // --- preconditioned by a general operator z = M r (AMG) -------------------
 
-// x = 0, r = b, partial b.b (scalars set by k_rz_start)
+// x = 0, r = b, p = 0 (rz = 0: the first iteration takes p = z), b.b.  With
+// sinv0 set, also the first sweep of the AMG V-cycle from zero (see
+// k_update_m).  n_done = NULL: the caller's next kernel decides who is done.
 __global__ void __launch_bounds__(NT) k_init_m(const double *__restrict__ b, double *__restrict__ x,
-                                               double *__restrict__ r, Tiles tl, double *partials,
-                                               unsigned *counter, KrylovScalars *ks, double rtol, int maxit) {
+                                               double *__restrict__ r, double *__restrict__ p, Tiles tl,
+                                               double *partials, unsigned *counter, KrylovScalars *ks, int *n_done,
+                                               double rtol, int maxit, const double *__restrict__ sinv0,
+                                               double *__restrict__ t0, double omega) {
   const int t = blockIdx.x;
   const int sys = tl.sys[t];
   const int r0 = tl.row0[t], r1 = tl.row1[t];
@@ -183,6 +193,8 @@ __global__ void __launch_bounds__(NT) k_init_m(const double *__restrict__ b, dou
     const double bi = b[i];
     x[i] = 0.0;
     r[i] = bi;
+    p[i] = 0.0;
+    if (sinv0) t0[i] = omega * sinv0[i] * bi;
     bb = fma(bi, bi, bb);
   }
   double v[1] = {bb}, out[1];
@@ -196,34 +208,10 @@ __global__ void __launch_bounds__(NT) k_init_m(const double *__restrict__ b, dou
     k.breakdown = 0;
     k.stalled = 0;
     k.inner_total = 0;
+    k.rz = 0.0;
     k.beta = 0.0;
     k.done = 0;
-  }
-}
-
-// p = z, rz = r.z; done if r.r already meets the tolerance (or the system is
-// done for another reason)
-__global__ void __launch_bounds__(NT) k_rz_start(const double *__restrict__ r, const double *__restrict__ z,
-                                                 double *__restrict__ p, Tiles tl, double *partials,
-                                                 unsigned *counter, KrylovScalars *ks, int *n_done) {
-  const int t = blockIdx.x;
-  const int sys = tl.sys[t];
-  const int r0 = tl.row0[t], r1 = tl.row1[t];
-  double rz = 0.0;
-  for (int i = r0 + threadIdx.x; i < r1; i += NT) {
-    const double zi = z[i];
-    p[i] = zi;
-    rz = fma(r[i], zi, rz);
-  }
-  double v[1] = {rz}, out[1];
-  if (seg_sum<NT, 1>(v, partials, counter, tl, t, sys, out) && threadIdx.x == 0) {
-    KrylovScalars &k = ks[sys];
-    k.rz = out[0];
-    k.beta = 0.0;
-    const bool fin = k.rr <= k.tol2 || k.iter >= k.maxit || k.breakdown || k.stalled;
-    k.done = fin ? 1 : 0;
-    if (fin) atomicAdd(n_done, 1);
-    else if (!(out[0] > 0.0)) { k.breakdown = 1; k.done = 1; atomicAdd(n_done, 1); }
+    if (n_done && out[0] <= k.tol2) { k.done = 1; atomicAdd(n_done, 1); }
   }
 }
 
@@ -235,12 +223,13 @@ __global__ void __launch_bounds__(NT) k_update_m(double *__restrict__ x, double 
                                                  const double *__restrict__ p, const double *__restrict__ q, Tiles tl,
                                                  double *partials, unsigned *counter, KrylovScalars *ks, int *n_done,
                                                  const double *__restrict__ sinv0, double *__restrict__ t0,
-                                                 double omega) {
+                                                 double omega, cudaGraphConditionalHandle loop) {
   const int t = blockIdx.x;
   const int sys = tl.sys[t];
   const int r0 = tl.row0[t], r1 = tl.row1[t];
   pdl_wait();
   pdl_trigger();
+  if (t == 0 && threadIdx.x == 0) loop_end_check(loop, n_done, tl.n_sys);
   if (ks[sys].done) return;
   const double alpha = ks[sys].alpha;
   double rr = 0.0;
@@ -258,7 +247,7 @@ __global__ void __launch_bounds__(NT) k_update_m(double *__restrict__ x, double 
     k.iter += 1;
     bool fin = out[0] <= k.tol2 || k.iter >= k.maxit;
     if (!(out[0] == out[0])) { k.breakdown = 1; fin = true; }
-    if (fin) { k.done = 1; atomicAdd(n_done, 1); }
+    if (fin) { k.done = 1; loop_system_done(loop, n_done, tl.n_sys); }
   }
 }
 
@@ -278,7 +267,7 @@ __global__ void __launch_bounds__(NT) k_rz(const double *__restrict__ r, const d
   double v[1] = {rz}, out[1];
   if (seg_sum<NT, 1>(v, partials, counter, tl, t, sys, out) && threadIdx.x == 0) {
     KrylovScalars &k = ks[sys];
-    k.beta = out[0] / k.rz;
+    k.beta = k.rz > 0.0 ? out[0] / k.rz : 0.0;   // 0 in the first iteration (rz starts at 0)
     k.rz = out[0];
     if (!(out[0] > 0.0)) { k.breakdown = 1; k.done = 1; atomicAdd(n_done, 1); }
   }
@@ -296,10 +285,13 @@ __global__ void __launch_bounds__(NT) k_pdir_z(double *__restrict__ p, const dou
   for (int i = r0 + threadIdx.x; i < r1; i += NT) p[i] = fma(beta, p[i], z[i]);
 }
 
-// restart for the general preconditioner: r = b - A x and r.r
+// restart for the general preconditioner: r = b - A x, p = 0 and r.r (a
+// system done for another reason stays done)
 __global__ void __launch_bounds__(NT) k_restart_m(const double *__restrict__ b, const double *__restrict__ Ax,
-                                                  double *__restrict__ r, Tiles tl, double *partials,
-                                                  unsigned *counter, KrylovScalars *ks) {
+                                                  double *__restrict__ r, double *__restrict__ p, Tiles tl,
+                                                  double *partials, unsigned *counter, KrylovScalars *ks, int *n_done,
+                                                  const double *__restrict__ sinv0, double *__restrict__ t0,
+                                                  double omega) {
   const int t = blockIdx.x;
   const int sys = tl.sys[t];
   const int r0 = tl.row0[t], r1 = tl.row1[t];
@@ -307,10 +299,19 @@ __global__ void __launch_bounds__(NT) k_restart_m(const double *__restrict__ b, 
   for (int i = r0 + threadIdx.x; i < r1; i += NT) {
     const double ri = b[i] - Ax[i];
     r[i] = ri;
+    p[i] = 0.0;
+    if (sinv0) t0[i] = omega * sinv0[i] * ri;
     rr = fma(ri, ri, rr);
   }
   double v[1] = {rr}, out[1];
-  if (seg_sum<NT, 1>(v, partials, counter, tl, t, sys, out) && threadIdx.x == 0) ks[sys].rr = out[0];
+  if (seg_sum<NT, 1>(v, partials, counter, tl, t, sys, out) && threadIdx.x == 0) {
+    KrylovScalars &k = ks[sys];
+    k.rr = out[0];
+    k.rz = 0.0;
+    k.beta = 0.0;
+    k.done = (out[0] <= k.tol2 || k.iter >= k.maxit || k.breakdown || k.stalled) ? 1 : 0;
+    if (k.done) atomicAdd(n_done, 1);
+  }
 }
 
 __global__ void __launch_bounds__(NT) k_resid2(const double *__restrict__ b, const double *__restrict__ Ax, Tiles tl,
@@ -477,9 +478,11 @@ __global__ void __launch_bounds__(NT) k_bi_update(double *__restrict__ x, double
 
 // p = r + beta (p - omega v)
 __global__ void __launch_bounds__(NT) k_bi_pdir(double *__restrict__ p, const double *__restrict__ r,
-                                                const double *__restrict__ v, Tiles tl, const KrylovScalars *ks) {
+                                                const double *__restrict__ v, Tiles tl, const KrylovScalars *ks,
+                                                cudaGraphConditionalHandle loop, int *n_done) {
   const int t = blockIdx.x;
   const int sys = tl.sys[t];
+  if (t == 0 && threadIdx.x == 0) loop_end_check(loop, n_done, tl.n_sys);
   if (ks[sys].done) return;
   const double beta = ks[sys].beta, omega = ks[sys].omega;
   for (int i = tl.row0[t] + threadIdx.x; i < tl.row1[t]; i += NT) p[i] = fma(beta, fma(-omega, v[i], p[i]), r[i]);
@@ -597,12 +600,12 @@ void ensure_krylov_buffers(System *s) {
   // per-system counters, one spare, then the group counters
   s->counter = sys_alloc<unsigned>(s, ns + 1 + s->seg.n_groups);
   s->ks = sys_alloc<KrylovScalars>(s, ns);
-  s->n_done = sys_alloc<int>(s, 1);
+  s->n_done = sys_alloc<int>(s, 2);
   s->u = sys_alloc<double>(s, (size_t)s->n_cv);
   VAG_CUDA(cudaMemsetAsync(s->counter, 0, (ns + 1 + s->seg.n_groups) * sizeof(unsigned), s->ctx->stream));
   VAG_CUDA(cudaMemsetAsync(s->u, 0, sizeof(double) * s->n_cv, s->ctx->stream));
   if (!s->ks_host) VAG_CUDA(cudaMallocHost(&s->ks_host, sizeof(KrylovScalars) * ns));
-  if (!s->n_done_host) VAG_CUDA(cudaMallocHost(&s->n_done_host, sizeof(int)));
+  if (!s->n_done_host) VAG_CUDA(cudaMallocHost(&s->n_done_host, 2 * sizeof(int)));
 }
 
 void launch_spmv_plain(System *s, const double *x, double *y, cudaStream_t st) { launch_spmv(s, x, y, 0, st); }
@@ -636,15 +639,26 @@ double time_spmv(System *s, int reps) {
   return (double)ms / reps;
 }
 
-static void pcg_iteration_amg(System *s, cudaStream_t st) {
+// Jacobi iterations per pass over their loop's body
+constexpr int kLoopUnroll = 4;
+
+// Kernels of the passes over a loop's body so far (System::n_done[1]), for
+// the launch count.  Waits for the loop.
+static void note_loop(System *s, const LoopGraph &g) {
+  VAG_CUDA(cudaMemcpyAsync(s->n_done_host, s->n_done, 2 * sizeof(int), cudaMemcpyDeviceToHost, s->ctx->stream));
+  VAG_CUDA(cudaStreamSynchronize(s->ctx->stream));
+  note_launches((unsigned long long)s->n_done_host[1] * g.nodes);
+}
+
+// One iteration of CG with the V-cycle, from r (and its first sweep t0) to
+// the next r: z = V(r) with r.z, p = z + beta p, q = A p with p.q, the update.
+// The convergence test is its last kernel, so that no V-cycle runs after it.
+static void pcg_iteration_amg(System *s, cudaStream_t st, cudaGraphConditionalHandle loop) {
   const Tiles tl = tiles_of(s);
   const int nt = s->seg.n_tiles;
-  launch_spmv(s, s->kp, s->kq, 1, st);
   double *t0 = nullptr;
   double omega = 0.0;
   const double *sinv0 = amg_first_sweep_scale(s, t0, omega);
-  launch_pdl(k_update_m, nt, NT, 0, st, s->kx, s->kr, (const double *)s->kp, (const double *)s->kq, tl, s->partials,
-             s->counter, s->ks, s->n_done, sinv0, t0, omega);
   const bool rz_done = sinv0 ? amg_apply_cg(s, s->kr, s->kz, st) : (amg_apply(s, s->kr, s->kz, st), false);
   if (!rz_done) {
     launch_pdl(k_rz, nt, NT, 0, st, (const double *)s->kr, (const double *)s->kz, tl, s->partials, s->counter, s->ks,
@@ -652,29 +666,33 @@ static void pcg_iteration_amg(System *s, cudaStream_t st) {
     note_launches(1);
   }
   launch_pdl(k_pdir_z, nt, NT, 0, st, s->kp, (const double *)s->kz, tl, (const KrylovScalars *)s->ks);
+  launch_spmv(s, s->kp, s->kq, 1, st);
+  launch_pdl(k_update_m, nt, NT, 0, st, s->kx, s->kr, (const double *)s->kp, (const double *)s->kq, tl, s->partials,
+             s->counter, s->ks, s->n_done, sinv0, t0, omega, loop);
   note_launches(2);
 }
 
-static void pcg_iteration(System *s, cudaStream_t st) {
+// check: this iteration ends a pass over the body of `loop`
+static void pcg_iteration(System *s, cudaStream_t st, bool check = false, cudaGraphConditionalHandle loop = 0) {
   const Tiles tl = tiles_of(s);
   launch_spmv(s, s->kp, s->kq, 1, st);
-  k_update<<<s->seg.n_tiles, NT, 0, st>>>(s->kx, s->kr, s->kp, s->kq, s->dinv, tl, s->partials, s->counter, s->ks,
-                                          s->n_done);
-  note_launches(1);
-  k_pdir<<<s->seg.n_tiles, NT, 0, st>>>(s->kp, s->kr, s->dinv, tl, s->ks);
-  note_launches(1);
+  launch_pdl(k_update, s->seg.n_tiles, NT, 0, st, s->kx, s->kr, (const double *)s->kp, (const double *)s->kq,
+             (const double *)s->dinv, tl, s->partials, s->counter, s->ks, s->n_done);
+  launch_pdl(k_pdir, s->seg.n_tiles, NT, 0, st, s->kp, (const double *)s->kr, (const double *)s->dinv, tl,
+             (const KrylovScalars *)s->ks, (int)check, loop, s->n_done);
+  note_launches(2);
 }
 
 // Chebyshev: the CG update also forms w = D^-1 r (the polynomial's first
 // step), the remaining steps follow, the last one forming r.z and beta
-static void pcg_iteration_cheb(System *s, cudaStream_t st) {
+static void pcg_iteration_cheb(System *s, cudaStream_t st, cudaGraphConditionalHandle loop) {
   const Tiles tl = tiles_of(s);
   const int nt = s->seg.n_tiles;
-  launch_spmv(s, s->kp, s->kq, 1, st);
-  launch_pdl(k_update_m, nt, NT, 0, st, s->kx, s->kr, (const double *)s->kp, (const double *)s->kq, tl, s->partials,
-             s->counter, s->ks, s->n_done, (const double *)s->dinv, s->cw, 1.0);
   cheb_apply(s, s->kr, s->kz, st, true, true, true);
   launch_pdl(k_pdir_z, nt, NT, 0, st, s->kp, (const double *)s->kz, tl, (const KrylovScalars *)s->ks);
+  launch_spmv(s, s->kp, s->kq, 1, st);
+  launch_pdl(k_update_m, nt, NT, 0, st, s->kx, s->kr, (const double *)s->kp, (const double *)s->kq, tl, s->partials,
+             s->counter, s->ks, s->n_done, (const double *)s->dinv, s->cw, 1.0, loop);
   note_launches(2);
 }
 
@@ -729,64 +747,51 @@ void pcg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     VAG_CUDA(cudaEventSynchronize(s->ev1));
     cudaEventElapsedTime(&setup_ms, s->ev0, s->ev1);
   }
-  auto apply_m = [&](const double *r, double *z) {
-    if (amg) amg_apply(s, r, z, st);
-    else cheb_apply(s, r, z, st, false, false, false);
-  };
-  VAG_CUDA(cudaMemsetAsync(s->n_done, 0, sizeof(int), st));
-  if (general) {
-    k_init_m<<<nt, NT, 0, st>>>(s->rhs, s->kx, s->kr, tl, s->partials, s->counter, s->ks, o->rtol, o->maxit);
-    apply_m(s->kr, s->kz);
-    k_rz_start<<<nt, NT, 0, st>>>(s->kr, s->kz, s->kp, tl, s->partials, s->counter, s->ks, s->n_done);
-    note_launches(2);
-  } else {
+  // the first step of the preconditioner, formed where r is (the V-cycle's
+  // first sweep, the polynomial's first step)
+  double *t0 = nullptr;
+  double omega = 0.0;
+  const double *sinv0 = nullptr;
+  if (amg) {
+    sinv0 = amg_first_sweep_scale(s, t0, omega);
+  } else if (cheb) {
+    sinv0 = s->dinv;
+    t0 = s->cw;
+    omega = 1.0;
+  }
+  VAG_CUDA(cudaMemsetAsync(s->n_done, 0, 2 * sizeof(int), st));
+  if (general)
+    k_init_m<<<nt, NT, 0, st>>>(s->rhs, s->kx, s->kr, s->kp, tl, s->partials, s->counter, s->ks, s->n_done, o->rtol,
+                                o->maxit, sinv0, t0, omega);
+  else
     k_init<<<nt, NT, 0, st>>>(s->rhs, s->dinv, s->kx, s->kr, s->kp, tl, s->partials, s->counter, s->ks,
                               s->n_done, o->rtol, o->maxit);
-    note_launches(1);
-  }
+  note_launches(1);
   VAG_CHECK_LAUNCH();
-  trace_mark(st, "CG start (r0, z0)");
-  const int chunk = 16;
-  cudaGraphExec_t &gexec = amg ? s->pcg_graph_amg : cheb ? s->pcg_graph_cheb : s->pcg_graph;
-  if (amg && gexec) {   // the hierarchy (and its pointers) is rebuilt every solve
-    cudaGraphExecDestroy(gexec);
-    gexec = nullptr;
+  trace_mark(st, "CG start (r0)");
+  // The iterations run in a loop that the device ends (kLoopUnroll of them a
+  // pass for Jacobi, whose three short kernels return at once when done).
+  LoopGraph &loop = amg ? s->pcg_loop_amg : cheb ? s->pcg_loop_cheb : s->pcg_loop;
+  if (amg || !loop.exec) {   // the hierarchy (and its pointers) is rebuilt every solve
+    loop_build(loop, st, [&](cudaGraphConditionalHandle h) {
+      if (amg) {
+        pcg_iteration_amg(s, st, h);
+      } else if (cheb) {
+        pcg_iteration_cheb(s, st, h);
+      } else {
+        for (int i = 0; i < kLoopUnroll; ++i) pcg_iteration(s, st, i + 1 == kLoopUnroll, h);
+      }
+    });
+    trace_mark(st, "loop capture + instantiate");
   }
-  if (!gexec) {
-    cudaGraph_t graph;
-    VAG_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    set_capturing(true);
-    for (int i = 0; i < chunk; ++i) {
-      if (amg) pcg_iteration_amg(s, st);
-      else if (cheb) pcg_iteration_cheb(s, st);
-      else pcg_iteration(s, st);
-    }
-    set_capturing(false);
-    VAG_CUDA(cudaStreamEndCapture(st, &graph));
-    size_t nodes = 0;
-    cudaGraphGetNodes(graph, nullptr, &nodes);
-    VAG_CUDA(cudaGraphInstantiate(&gexec, graph, 0));
-    cudaGraphDestroy(graph);
-    if (amg) s->amg_graph_nodes = nodes;
-    if (cheb) s->cheb_graph_nodes = nodes;
-    trace_mark(st, "graph capture + instantiate");
-  }
-  const unsigned long long per_launch = amg ? s->amg_graph_nodes : cheb ? s->cheb_graph_nodes : 3ull * chunk;
-  const int max_chunks = (o->maxit + chunk - 1) / chunk;
   // The recursive residual can drift below the true one; after convergence
   // the true residual is recomputed and CG restarts from the current iterate
   // (a few times at most) for every system still above its tolerance whose
   // true residual still falls.
   std::vector<double> prev_res2;
   for (int attempt = 0;; ++attempt) {
-    for (int c = 0; c < max_chunks + 1; ++c) {
-      VAG_CUDA(cudaMemcpyAsync(s->n_done_host, s->n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
-      VAG_CUDA(cudaStreamSynchronize(st));
-      if (*s->n_done_host >= ns) break;
-      VAG_CUDA(cudaGraphLaunch(gexec, st));
-      note_launches(per_launch);
-    }
-    trace_mark(st, "CG iterations (graph chunks)");
+    VAG_CUDA(cudaGraphLaunch(loop.exec, st));
+    trace_mark(st, "CG iterations");
     launch_spmv(s, s->kx, s->kq, 0, st);
     k_resid2<<<nt, NT, 0, st>>>(s->rhs, s->kq, tl, s->partials, s->counter, s->ks);
     note_launches(1);
@@ -808,17 +813,16 @@ void pcg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     // push the stall flags back before the restart kernels read them
     VAG_CUDA(cudaMemcpyAsync(s->ks, s->ks_host, sizeof(KrylovScalars) * ns, cudaMemcpyHostToDevice, st));
     VAG_CUDA(cudaMemsetAsync(s->n_done, 0, sizeof(int), st));
-    if (general) {
-      k_restart_m<<<nt, NT, 0, st>>>(s->rhs, s->kq, s->kr, tl, s->partials, s->counter, s->ks);
-      apply_m(s->kr, s->kz);
-      k_rz_start<<<nt, NT, 0, st>>>(s->kr, s->kz, s->kp, tl, s->partials, s->counter, s->ks, s->n_done);
-      note_launches(2);
-    } else {
+    if (general)
+      k_restart_m<<<nt, NT, 0, st>>>(s->rhs, s->kq, s->kr, s->kp, tl, s->partials, s->counter, s->ks, s->n_done,
+                                     sinv0, t0, omega);
+    else
       k_restart<<<nt, NT, 0, st>>>(s->rhs, s->kq, s->dinv, s->kr, s->kp, tl, s->partials, s->counter, s->ks,
                                    s->n_done);
-      note_launches(1);
-    }
+    note_launches(1);
+    VAG_CHECK_LAUNCH();
   }
+  note_loop(s, loop);
   finish_solve(s, info, false);
   info->ms_setup = setup_ms;
   info->ms_solve -= setup_ms;
@@ -863,22 +867,15 @@ void bicgstab_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
       note_launches(1);
     }
   };
-  VAG_CUDA(cudaMemsetAsync(s->n_done, 0, sizeof(int), st));
-  k_init_m<<<nt, NT, 0, st>>>(s->rhs, s->kx, s->kr, tl, s->partials, s->counter, s->ks, o->rtol, o->maxit);
+  VAG_CUDA(cudaMemsetAsync(s->n_done, 0, 2 * sizeof(int), st));
+  k_init_m<<<nt, NT, 0, st>>>(s->rhs, s->kx, s->kr, s->kp, tl, s->partials, s->counter, s->ks, nullptr, o->rtol,
+                              o->maxit, nullptr, nullptr, 0.0);
   k_bi_start<<<nt, NT, 0, st>>>(s->kr, s->b_r0, s->kp, tl, s->ks, s->n_done);
   note_launches(2);
   VAG_CHECK_LAUNCH();
-  // iterations in a CUDA graph of `chunk` iterations, rebuilt every solve
-  // (the AMG hierarchy's buffers are new each time)
-  const int chunk = 8;
-  if (s->bicg_graph) {
-    cudaGraphExecDestroy(s->bicg_graph);
-    s->bicg_graph = nullptr;
-  }
-  cudaGraph_t graph;
-  VAG_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-  set_capturing(true);
-  for (int i = 0; i < chunk; ++i) {
+  // iterations in a loop that the device ends, rebuilt every solve (the AMG
+  // hierarchy's buffers are new each time)
+  loop_build(s->bicg_loop, st, [&](cudaGraphConditionalHandle h) {
     precond(s->kp, s->b_ph);
     launch_spmv(s, s->b_ph, s->kq, 0, st);   // v
     k_bi_alpha<<<nt, NT, 0, st>>>(s->b_r0, s->kq, tl, s->partials, s->counter, s->ks, s->n_done);
@@ -888,24 +885,11 @@ void bicgstab_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     k_bi_omega<<<nt, NT, 0, st>>>(s->b_t, s->b_s, tl, s->partials, s->counter, s->ks);
     k_bi_update<<<nt, NT, 0, st>>>(s->kx, s->kr, s->b_ph, s->b_sh, s->b_s, s->b_t, s->b_r0, tl, s->partials,
                                    s->counter, s->ks, s->n_done);
-    k_bi_pdir<<<nt, NT, 0, st>>>(s->kp, s->kr, s->kq, tl, s->ks);
+    k_bi_pdir<<<nt, NT, 0, st>>>(s->kp, s->kr, s->kq, tl, s->ks, h, s->n_done);
     note_launches(5);
-  }
-  set_capturing(false);
-  VAG_CUDA(cudaStreamEndCapture(st, &graph));
-  size_t nodes = 0;
-  cudaGraphGetNodes(graph, nullptr, &nodes);
-  VAG_CUDA(cudaGraphInstantiate(&s->bicg_graph, graph, 0));
-  cudaGraphDestroy(graph);
-  const int ns = s->seg.n_sys;
-  const int max_chunks = (o->maxit + chunk - 1) / chunk;
-  for (int c = 0; c < max_chunks + 1; ++c) {
-    VAG_CUDA(cudaMemcpyAsync(s->n_done_host, s->n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
-    VAG_CUDA(cudaStreamSynchronize(st));
-    if (*s->n_done_host >= ns) break;
-    VAG_CUDA(cudaGraphLaunch(s->bicg_graph, st));
-    note_launches(nodes);
-  }
+  });
+  VAG_CUDA(cudaGraphLaunch(s->bicg_loop.exec, st));
+  note_loop(s, s->bicg_loop);
   // the true residual decides the status
   launch_spmv(s, s->kx, s->kq, 0, st);
   k_resid2<<<nt, NT, 0, st>>>(s->rhs, s->kq, tl, s->partials, s->counter, s->ks);

@@ -112,9 +112,11 @@ __global__ void __launch_bounds__(NT) k_upd32(float *__restrict__ x, float *__re
 }
 
 __global__ void __launch_bounds__(NT) k_pdir32(float *__restrict__ p, const float *__restrict__ r, Tiles tl,
-                                               const KrylovScalars *ks) {
+                                               const KrylovScalars *ks, int check, cudaGraphConditionalHandle loop,
+                                               int *n_done) {
   const int t = blockIdx.x;
   const int sys = tl.sys[t];
+  if (check && t == 0 && threadIdx.x == 0) loop_end_check(loop, n_done, tl.n_sys);
   if (ks[sys].done) return;
   const float b = (float)ks[sys].beta;
   const int r0 = tl.row0[t], r1 = tl.row1[t];
@@ -289,11 +291,15 @@ __global__ void __launch_bounds__(NT) k_spmv32d(const int *__restrict__ rowptr, 
   }
 }
 
-// r32 = r / ||r|| (per system), x32 = 0; inner scalars and tolerance
+// r32 = r / ||r|| (per system), x32 = p32 = 0 (rz = 0: the first iteration
+// takes p = z), with sinv0 set the V-cycle's first sweep from zero; inner
+// scalars and tolerance
 __global__ void __launch_bounds__(NT) k_irm_prep(const double *__restrict__ r, float *__restrict__ r32,
-                                                 float *__restrict__ x32, Tiles tl, double *partials,
-                                                 unsigned *counter, const KrylovScalars *ko, KrylovScalars *ki,
-                                                 int *n_done_in, double eta_min, int maxit_in) {
+                                                 float *__restrict__ x32, float *__restrict__ p32, Tiles tl,
+                                                 double *partials, unsigned *counter, const KrylovScalars *ko,
+                                                 KrylovScalars *ki, int *n_done_in, double eta_min, int maxit_in,
+                                                 const float *__restrict__ sinv0, float *__restrict__ t0,
+                                                 float omega) {
   const int t = blockIdx.x;
   const int sys = tl.sys[t];
   const bool outer_done = ko[sys].done;
@@ -305,6 +311,8 @@ __global__ void __launch_bounds__(NT) k_irm_prep(const double *__restrict__ r, f
       const float v = (float)(r[i] * inv);
       r32[i] = v;
       x32[i] = 0.f;
+      p32[i] = 0.f;
+      if (sinv0) t0[i] = omega * sinv0[i] * v;
       rr = fmaf(v, v, rr);
     }
   }
@@ -327,45 +335,19 @@ __global__ void __launch_bounds__(NT) k_irm_prep(const double *__restrict__ r, f
   }
 }
 
-// p32 = z32, rz = r.z (breakdown unless positive)
-__global__ void __launch_bounds__(NT) k_irm_rz_start(const float *__restrict__ r, const float *__restrict__ z,
-                                                     float *__restrict__ p, Tiles tl, double *partials,
-                                                     unsigned *counter, KrylovScalars *ki, int *n_done_in) {
-  const int t = blockIdx.x;
-  const int sys = tl.sys[t];
-  pdl_wait();
-  pdl_trigger();
-  if (ki[sys].done) return;
-  const int r0 = tl.row0[t], r1 = tl.row1[t];
-  float rz = 0.f;
-  for (int i = r0 + threadIdx.x; i < r1; i += NT) {
-    const float zi = z[i];
-    p[i] = zi;
-    rz = fmaf(r[i], zi, rz);
-  }
-  double v[1] = {(double)rz}, out[1];
-  if (seg_sum<NT, 1>(v, partials, counter, tl, t, sys, out) && threadIdx.x == 0) {
-    KrylovScalars &k = ki[sys];
-    k.rz = out[0];
-    if (!(out[0] > 0.0)) {
-      k.breakdown = 1;
-      k.done = 1;
-      atomicAdd(n_done_in, 1);
-    }
-  }
-}
-
 // x += alpha p, r -= alpha q, r.r; the last tile counts the iteration and
 // tests the inner tolerance
 __global__ void __launch_bounds__(NT) k_irm_update(float *__restrict__ x, float *__restrict__ r,
                                                    const float *__restrict__ p, const float *__restrict__ q, Tiles tl,
                                                    double *partials, unsigned *counter, KrylovScalars *ki,
                                                    int *n_done_in, const float *__restrict__ sinv0,
-                                                   float *__restrict__ t0, float omega) {
+                                                   float *__restrict__ t0, float omega,
+                                                   cudaGraphConditionalHandle loop) {
   const int t = blockIdx.x;
   const int sys = tl.sys[t];
   pdl_wait();
   pdl_trigger();
+  if (t == 0 && threadIdx.x == 0) loop_end_check(loop, n_done_in, tl.n_sys);
   if (ki[sys].done) return;
   const float a = (float)ki[sys].alpha;
   const int r0 = tl.row0[t], r1 = tl.row1[t];
@@ -385,12 +367,12 @@ __global__ void __launch_bounds__(NT) k_irm_update(float *__restrict__ x, float 
     if (out[0] <= k.tol2 || k.iter >= k.maxit || !(out[0] == out[0])) {
       if (!(out[0] == out[0])) k.breakdown = 1;
       k.done = 1;
-      atomicAdd(n_done_in, 1);
+      loop_system_done(loop, n_done_in, tl.n_sys);
     }
   }
 }
 
-// beta = (r.z)_new / (r.z)_old
+// beta = (r.z)_new / (r.z)_old (0 in the first iteration, where rz is 0)
 __global__ void __launch_bounds__(NT) k_irm_rz(const float *__restrict__ r, const float *__restrict__ z, Tiles tl,
                                                double *partials, unsigned *counter, KrylovScalars *ki,
                                                int *n_done_in) {
@@ -405,7 +387,7 @@ __global__ void __launch_bounds__(NT) k_irm_rz(const float *__restrict__ r, cons
   double v[1] = {(double)rz}, out[1];
   if (seg_sum<NT, 1>(v, partials, counter, tl, t, sys, out) && threadIdx.x == 0) {
     KrylovScalars &k = ki[sys];
-    k.beta = out[0] / k.rz;
+    k.beta = k.rz > 0.0 ? out[0] / k.rz : 0.0;
     k.rz = out[0];
     if (!(out[0] > 0.0)) {
       k.breakdown = 1;
@@ -456,7 +438,22 @@ static void ensure_ir_vectors(System *s) {
   s->mx.p32 = sys_alloc<float>(s, n);
   s->mx.q32 = sys_alloc<float>(s, n);
   s->mx.ks_in = sys_alloc<KrylovScalars>(s, ns);
-  s->mx.n_done_in = sys_alloc<int>(s, 1);
+  s->mx.n_done_in = sys_alloc<int>(s, 2);
+}
+
+// Jacobi iterations per pass over their loop's body
+constexpr int kLoopUnroll = 4;
+
+// Waits for a refinement step and returns whether every system is done; the
+// kernels of the step's inner loop go to the launch count.
+static bool poll(System *s, int outer, const LoopGraph &inner) {
+  cudaStream_t st = s->ctx->stream;
+  VAG_CUDA(cudaMemcpyAsync(&s->n_done_host[0], s->n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
+  if (outer)
+    VAG_CUDA(cudaMemcpyAsync(&s->n_done_host[1], s->mx.n_done_in + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaStreamSynchronize(st));
+  if (outer) note_launches((unsigned long long)s->n_done_host[1] * inner.nodes);
+  return s->n_done_host[0] >= s->seg.n_sys;
 }
 
 static void ensure_mixed_buffers(System *s) {
@@ -488,38 +485,23 @@ void mixed_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
                                kMaxOuter);
   note_launches(1);
   VAG_CHECK_LAUNCH();
-  const int chunk = 16;
-  if (!m.graph) {
-    cudaGraph_t graph;
-    VAG_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    set_capturing(true);
-    for (int i = 0; i < chunk; ++i) {
-      spmv32<<<nt, NT, 0, st>>>(s->rowptr, s->slice_ptr, s->scol, m.sval32, m.p32, m.q32, tl, s->partials,
-                                s->counter, m.ks_in, m.n_done_in);
-      k_upd32<<<nt, NT, 0, st>>>(m.x32, m.r32, m.p32, m.q32, tl, s->partials, s->counter, m.ks_in, m.n_done_in);
-      k_pdir32<<<nt, NT, 0, st>>>(m.p32, m.r32, tl, m.ks_in);
-    }
-    set_capturing(false);
-    VAG_CUDA(cudaStreamEndCapture(st, &graph));
-    VAG_CUDA(cudaGraphInstantiate(&m.graph, graph, 0));
-    cudaGraphDestroy(graph);
-  }
+  if (!m.loop.exec)
+    loop_build(m.loop, st, [&](cudaGraphConditionalHandle h) {
+      for (int i = 0; i < kLoopUnroll; ++i) {
+        spmv32<<<nt, NT, 0, st>>>(s->rowptr, s->slice_ptr, s->scol, m.sval32, m.p32, m.q32, tl, s->partials,
+                                  s->counter, m.ks_in, m.n_done_in);
+        k_upd32<<<nt, NT, 0, st>>>(m.x32, m.r32, m.p32, m.q32, tl, s->partials, s->counter, m.ks_in, m.n_done_in);
+        k_pdir32<<<nt, NT, 0, st>>>(m.p32, m.r32, tl, m.ks_in, i + 1 == kLoopUnroll, h, m.n_done_in);
+      }
+    });
   int outer = 0;
   for (; outer < kMaxOuter + 1; ++outer) {
-    VAG_CUDA(cudaMemcpyAsync(s->n_done_host, s->n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
-    VAG_CUDA(cudaStreamSynchronize(st));
-    if (*s->n_done_host >= ns) break;
-    VAG_CUDA(cudaMemsetAsync(m.n_done_in, 0, sizeof(int), st));
+    if (poll(s, outer, m.loop)) break;
+    VAG_CUDA(cudaMemsetAsync(m.n_done_in, 0, 2 * sizeof(int), st));
     k_ir_prep<<<nt, NT, 0, st>>>(s->kr, m.sc, m.r32, m.x32, m.p32, tl, s->partials, s->counter, s->ks, m.ks_in,
                                  m.n_done_in, kEta, o->maxit);
     note_launches(1);
-    for (int c = 0; c < (o->maxit + chunk - 1) / chunk + 1; ++c) {
-      VAG_CUDA(cudaMemcpyAsync(s->n_done_host, m.n_done_in, sizeof(int), cudaMemcpyDeviceToHost, st));
-      VAG_CUDA(cudaStreamSynchronize(st));
-      if (*s->n_done_host >= ns) break;
-      VAG_CUDA(cudaGraphLaunch(m.graph, st));
-      note_launches(3ull * chunk);
-    }
+    VAG_CUDA(cudaGraphLaunch(m.loop.exec, st));
     k_ir_correct<<<nt, NT, 0, st>>>(s->kx, m.x32, m.sc, tl, s->ks);
     note_launches(1);
     spmv_f64(s, s->kx, s->kq);
@@ -561,72 +543,43 @@ void mixed_amg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   cudaEventElapsedTime(&setup_ms, s->ev0, s->ev1);
   const float *a32 = m.dval32;   // FP32 difference-form values of A, sliced ELL
   auto spmv32 = s->sell_u == 2 ? k_spmv32d<2> : s->sell_u == 8 ? k_spmv32d<8> : k_spmv32d<4>;
-  // one inner iteration: q = A p (p.q, alpha), x/r update, z = V(r), r.z, p
-  // the V-cycle's first sweep is formed by the update and its last sweep
-  // forms r.z (the same arithmetic as the separate kernels)
+  // one inner iteration, from r (and the V-cycle's first sweep) to the next r:
+  // z = V(r) with r.z, p = z + beta p, q = A p with p.q, the update, which
+  // forms the next first sweep and tests the inner tolerance (so that no
+  // V-cycle runs after the last iteration)
   float *t0 = nullptr;
   float omega = 0.f;
   const float *sinv0 = amg_first_sweep_scale_f32(s, t0, omega);
-  auto iteration = [&]() {
+  auto iteration = [&](cudaGraphConditionalHandle loop) {
+    const bool rz_done = sinv0 ? amg_apply_f32_cg(s, m.r32, m.z32, st, m.ks_in, m.n_done_in)
+                               : (amg_apply_f32(s, m.r32, m.z32, st), false);
+    if (!rz_done)
+      launch_pdl(k_irm_rz, nt, NT, 0, st, (const float *)m.r32, (const float *)m.z32, tl, s->partials, s->counter,
+                 m.ks_in, m.n_done_in);
+    launch_pdl(k_irm_pdir, nt, NT, 0, st, m.p32, (const float *)m.z32, tl, (const KrylovScalars *)m.ks_in);
     launch_pdl(spmv32, nt, NT, 0, st, (const int *)s->rowptr, (const int *)s->slice_ptr, (const int *)s->scol, a32,
                (const float *)m.rowsum32, (const float *)m.p32, m.q32, tl, s->partials, s->counter, m.ks_in,
                m.n_done_in);
     launch_pdl(k_irm_update, nt, NT, 0, st, m.x32, m.r32, (const float *)m.p32, (const float *)m.q32, tl, s->partials,
-               s->counter, m.ks_in, m.n_done_in, sinv0, t0, omega);
-    const bool rz_done = sinv0 ? amg_apply_f32_cg(s, m.r32, m.z32, st, m.ks_in, m.n_done_in)
-                               : (amg_apply_f32(s, m.r32, m.z32, st), false);
-    if (!rz_done) {
-      launch_pdl(k_irm_rz, nt, NT, 0, st, (const float *)m.r32, (const float *)m.z32, tl, s->partials, s->counter,
-                 m.ks_in, m.n_done_in);
-      note_launches(1);
-    }
-    launch_pdl(k_irm_pdir, nt, NT, 0, st, m.p32, (const float *)m.z32, tl, (const KrylovScalars *)m.ks_in);
-    note_launches(3);
+               s->counter, m.ks_in, m.n_done_in, sinv0, t0, omega, loop);
   };
   VAG_CUDA(cudaMemsetAsync(s->n_done, 0, sizeof(int), st));
   k_ir_init<<<nt, NT, 0, st>>>(s->rhs, s->kx, s->kr, tl, s->partials, s->counter, s->ks, s->n_done, o->rtol,
                                kMaxOuter);
   note_launches(1);
   VAG_CHECK_LAUNCH();
-  // the hierarchy is rebuilt every solve, so is the graph of inner iterations
-  const int chunk = 8;
-  if (m.graph_amg) {
-    cudaGraphExecDestroy(m.graph_amg);
-    m.graph_amg = nullptr;
-  }
-  {
-    cudaGraph_t graph;
-    VAG_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-    set_capturing(true);
-    for (int i = 0; i < chunk; ++i) iteration();
-    set_capturing(false);
-    VAG_CUDA(cudaStreamEndCapture(st, &graph));
-    cudaGraphGetNodes(graph, nullptr, &m.graph_amg_nodes);
-    VAG_CUDA(cudaGraphInstantiate(&m.graph_amg, graph, 0));
-    cudaGraphDestroy(graph);
-    trace_mark(st, "graph capture + instantiate");
-  }
+  // the hierarchy is rebuilt every solve, so is the loop of inner iterations
+  loop_build(m.loop_amg, st, iteration);
+  trace_mark(st, "loop capture + instantiate");
   const double eta_min = o->inner_rtol > 0.0 ? o->inner_rtol : kEtaAmg;
   for (int outer = 0; outer < kMaxOuter + 1; ++outer) {
-    VAG_CUDA(cudaMemcpyAsync(s->n_done_host, s->n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
-    VAG_CUDA(cudaStreamSynchronize(st));
-    if (*s->n_done_host >= ns) break;
-    VAG_CUDA(cudaMemsetAsync(m.n_done_in, 0, sizeof(int), st));
-    k_irm_prep<<<nt, NT, 0, st>>>(s->kr, m.r32, m.x32, tl, s->partials, s->counter, s->ks, m.ks_in, m.n_done_in,
-                                  eta_min, o->maxit);
-    note_launches(1);
-    amg_apply_f32(s, m.r32, m.z32, st);
-    launch_pdl(k_irm_rz_start, nt, NT, 0, st, (const float *)m.r32, (const float *)m.z32, m.p32, tl, s->partials,
-               s->counter, m.ks_in, m.n_done_in);
+    if (poll(s, outer, m.loop_amg)) break;
+    VAG_CUDA(cudaMemsetAsync(m.n_done_in, 0, 2 * sizeof(int), st));
+    k_irm_prep<<<nt, NT, 0, st>>>(s->kr, m.r32, m.x32, m.p32, tl, s->partials, s->counter, s->ks, m.ks_in, m.n_done_in,
+                                  eta_min, o->maxit, sinv0, t0, omega);
     note_launches(1);
     VAG_CHECK_LAUNCH();
-    for (int c = 0; c < (o->maxit + chunk - 1) / chunk + 1; ++c) {
-      VAG_CUDA(cudaMemcpyAsync(s->n_done_host, m.n_done_in, sizeof(int), cudaMemcpyDeviceToHost, st));
-      VAG_CUDA(cudaStreamSynchronize(st));
-      if (*s->n_done_host >= ns) break;
-      VAG_CUDA(cudaGraphLaunch(m.graph_amg, st));
-      note_launches(m.graph_amg_nodes);
-    }
+    VAG_CUDA(cudaGraphLaunch(m.loop_amg.exec, st));
     k_irm_correct<<<nt, NT, 0, st>>>(s->kx, m.x32, tl, s->ks);
     note_launches(1);
     spmv_f64(s, s->kx, s->kq);
