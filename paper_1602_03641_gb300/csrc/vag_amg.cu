@@ -60,6 +60,7 @@ constexpr double kOmega = 4.0 / 3.0;
 constexpr int kDenseMax = 96;
 constexpr size_t kDenseSmem = 2 * sizeof(double) * kDenseMax * kDenseMax;   // [A | B] in dynamic shared memory
 constexpr int kMaxLevels = 16;
+constexpr int kDenseStatusPin = 8;  // pinned word of the terminal blocks' status
 constexpr int kCoarseWidth = 160;   // unique columns of one coarse row (< 256)
 
 constexpr unsigned long long KEY_IN = ~0ull;
@@ -120,10 +121,12 @@ __global__ void k_strength(int n, const int *__restrict__ rowptr, const int *__r
   state[i] = cnt ? 0 : -2;   // 0 undecided, 1 root, -1 out, -2 isolated
 }
 
-__global__ void k_skip_rows(int n, const int *__restrict__ sys_start, int n_sys, const uint8_t *__restrict__ term,
-                            uint8_t *skip) {
+// rows of the systems that end at this level (at most kDenseMax rows)
+__global__ void k_skip_rows(int n, const int *__restrict__ sys_start, int n_sys, uint8_t *skip) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) skip[i] = term[sys_of_row(i, sys_start, n_sys)];
+  if (i >= n) return;
+  const int g = sys_of_row(i, sys_start, n_sys);
+  skip[i] = sys_start[g + 1] - sys_start[g] <= kDenseMax;
 }
 
 __device__ __forceinline__ unsigned long long node_key(int i, int8_t st, const int *__restrict__ sys_start, int n_sys) {
@@ -1196,9 +1199,23 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
   A.levels.clear();
   s->ctx->in_use -= A.bytes;
   A.bytes = 0;
-  auto alloc = [&](size_t bytes) -> void * {
+  // small arrays share chunks: a hierarchy has a few hundred, most of a few KB
+  unsigned char *chunk = nullptr;
+  size_t chunk_left = 0;
+  std::function<void *(size_t)> alloc = [&](size_t bytes) -> void * {
+    constexpr size_t kSmall = 32 << 10, kChunk = 256 << 10;
     bytes = (bytes + 255) & ~size_t(255);
     if (!bytes) bytes = 256;
+    if (bytes <= kSmall) {
+      if (bytes > chunk_left) {
+        chunk = static_cast<unsigned char *>(alloc(kChunk));
+        chunk_left = kChunk;
+      }
+      void *p = chunk;
+      chunk += bytes;
+      chunk_left -= bytes;
+      return p;
+    }
     if (s->ctx->budget && s->ctx->in_use + bytes > s->ctx->budget) fail(VAG_EBUDGET, "AMG hierarchy exceeds the budget");
     void *p = ctx_alloc(s->ctx, bytes);
     A.allocs.push_back(p);
@@ -1222,10 +1239,9 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
   L0.sell_nnz = s->sell_nnz;
   A.levels.push_back(L0);
   int *undecided = static_cast<int *>(alloc(sizeof(int)));
-  if (!s->amg_pin) VAG_CUDA(cudaMallocHost(&s->amg_pin, 4 * sizeof(int)));
-  int *und_host = s->n_done_host;   // pinned int
-  std::vector<uint8_t> term(ns);
-  std::vector<long long> off(ns + 1);
+  int *pin = ctx_pin(s->ctx);
+  int *dense_status = s->status + 1;   // set by the inversions of the terminal blocks, read once at the end
+  VAG_CUDA(cudaMemsetAsync(dense_status, 0, sizeof(int), st));
   for (int lvl = 0;; ++lvl) {
     if (lvl == kMaxLevels) fail(VAG_ECUDA, "AMG: hierarchy deeper than the level cap");
     // systems that end here: at most kDenseMax rows at this level (a system
@@ -1234,33 +1250,30 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
       AmgLevel &L = A.levels[lvl];
       const int n = L.n;
       bool any = false, all = true;
-      off[0] = 0;
+      std::vector<long long> &off = L.inv_off_h;   // lives as long as the level: uploaded without a wait
+      off.assign(ns + 1, 0);
       for (int g = 0; g < ns; ++g) {
         const int m = L.sys_start[g + 1] - L.sys_start[g];
-        term[g] = m <= kDenseMax;
-        any |= term[g] && m > 0;
-        all &= term[g];
-        off[g + 1] = off[g] + (term[g] && m > 0 ? (long long)m * m : 0);
+        const bool term = m <= kDenseMax;
+        any |= term && m > 0;
+        all &= term;
+        off[g + 1] = off[g] + (term && m > 0 ? (long long)m * m : 0);
       }
       L.any_term = any;
       L.all_term = all;
       L.n_inv = off[ns];
-      uint8_t *dterm = static_cast<uint8_t *>(alloc(ns));
-      VAG_CUDA(cudaMemcpyAsync(dterm, term.data(), ns, cudaMemcpyHostToDevice, st));
       L.skip = static_cast<uint8_t *>(alloc(std::max(n, 1)));
-      k_skip_rows<<<grid_for(n, TB), TB, 0, st>>>(n, L.d_sys_start, ns, dterm, L.skip);
+      k_skip_rows<<<grid_for(n, TB), TB, 0, st>>>(n, L.d_sys_start, ns, L.skip);
       note_launches(1);
       if (any) {
         L.inv = static_cast<double *>(alloc(8 * (size_t)std::max<long long>(off[ns], 1)));
         L.inv_off = static_cast<long long *>(alloc(8 * ((size_t)ns + 1)));
         VAG_CUDA(cudaMemcpyAsync(L.inv_off, off.data(), 8 * (ns + 1), cudaMemcpyHostToDevice, st));
-        VAG_CUDA(cudaMemsetAsync(s->status, 0, sizeof(int), st));
         VAG_CUDA(cudaFuncSetAttribute(k_dense_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDenseSmem));
         k_dense_inverse<<<ns, TB, kDenseSmem, st>>>(L.d_sys_start, L.rowptr, L.col, L.val, L.inv_off, L.inv,
-                                                   s->status);
+                                                   dense_status);
         note_launches(1);
         VAG_CHECK_LAUNCH();
-        if (read_status(s) & ST_NONPOSITIVE) fail(VAG_EINVAL, "AMG: a terminal block is not positive definite");
       }
       if (all) break;
     }
@@ -1285,6 +1298,7 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
     trace_mark(st, "level: terminal blocks + strength");
     // MIS(2) rounds (state and next alternate), polled after 8 rounds and
     // then every 4 (a round after the last decision changes nothing)
+    int left = 0;
     for (int r = 0, poll = 8; r < 64;) {
       k_mis_max1<<<grid_for(n, TB), TB, 0, st>>>(n, L.rowptr, L.col, strong, state, L.d_sys_start, ns, m1,
                                                  undecided);
@@ -1293,18 +1307,19 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
       note_launches(2);
       std::swap(state, next);
       if (++r < poll && r < 64) continue;
-      VAG_CUDA(cudaMemcpyAsync(und_host, undecided, sizeof(int), cudaMemcpyDeviceToHost, st));
+      VAG_CUDA(cudaMemcpyAsync(pin, undecided, sizeof(int), cudaMemcpyDeviceToHost, st));
       VAG_CUDA(cudaStreamSynchronize(st));
-      if (*und_host == 0) break;
+      left = *pin;
+      if (left == 0) break;
       poll += 4;
     }
-    if (*und_host != 0) fail(VAG_ECUDA, "AMG: MIS(2) did not finish in 64 rounds");
+    if (left != 0) fail(VAG_ECUDA, "AMG: MIS(2) did not finish in 64 rounds");
     trace_mark(st, "level: MIS(2)");
     int *flag = static_cast<int *>(alloc(4 * (size_t)n));
     int *rscan = static_cast<int *>(alloc(4 * ((size_t)n + 1)));
     k_root_flags<<<grid_for(n, TB), TB, 0, st>>>(n, state, flag);
     note_launches(1);
-    const int nc = scan_exclusive(flag, rscan, n, st);
+    const int nc = scan_exclusive(s->ctx, flag, rscan, n);
     int *agg1 = static_cast<int *>(alloc(4 * (size_t)n));
     L.agg = static_cast<int *>(alloc(4 * (size_t)n));
     k_agg_pass1<<<grid_for(n, TB), TB, 0, st>>>(n, L.rowptr, L.col, strong, state, rscan, agg1);
@@ -1319,7 +1334,7 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
     VAG_CUDA(cudaMemsetAsync(cursor, 0, 4 * ((size_t)nc + 1), st));
     k_member_count<<<grid_for(n, TB), TB, 0, st>>>(n, L.agg, cnt);
     note_launches(1);
-    scan_exclusive(cnt, L.mptr, nc, st, false);   // at most n members: no need to wait for the total
+    scan_exclusive(s->ctx, cnt, L.mptr, nc, false);   // at most n members: no need to wait for the total
     L.mem = static_cast<int *>(alloc(4 * (size_t)std::max(n, 1)));
     k_member_fill<<<grid_for(n, TB), TB, 0, st>>>(n, L.agg, L.mptr, cursor, L.mem);
     k_sort_members<<<grid_for(nc, TB), TB, 0, st>>>(nc, L.mptr, L.mem);
@@ -1330,34 +1345,32 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
     C.n = nc;
     C.rowptr = static_cast<int *>(alloc(4 * ((size_t)nc + 1)));
     C.dinv = static_cast<double *>(alloc(8 * (size_t)std::max(nc, 1)));
-    int *tcol;
-    double *tval;
-    VAG_CUDA(cudaMallocAsync(&tcol, 4 * (size_t)std::max(nc, 1) * kCoarseWidth, st));
-    VAG_CUDA(cudaMallocAsync(&tval, 8 * (size_t)std::max(nc, 1) * kCoarseWidth, st));
+    Scratch scratch(s->ctx);
+    int *tcol = scratch.get<int>((size_t)nc * kCoarseWidth);
+    double *tval = scratch.get<double>((size_t)nc * kCoarseWidth);
     VAG_CUDA(cudaMemsetAsync(s->status, 0, sizeof(int), st));
     k_coarse_build<<<grid_for(nc, kBuildWarps), 32 * kBuildWarps, 0, st>>>(nc, L.mptr, L.mem, L.rowptr, L.col, L.val,
                                                                             L.agg, tcol, tval, cnt, C.dinv, s->status);
     note_launches(1);
-    scan_exclusive(cnt, C.rowptr, nc, st, false);
+    scan_exclusive(s->ctx, cnt, C.rowptr, nc, false);
     C.d_sys_start = static_cast<int *>(alloc(4 * ((size_t)ns + 1)));
     k_coarse_starts<<<grid_for(ns + 1, TB), TB, 0, st>>>(ns, L.d_sys_start, rscan, C.d_sys_start);
     note_launches(1);
     // one wait for the coarse nonzero count, the status and the row starts
-    C.sys_start.assign(ns + 1, 0);
-    VAG_CUDA(cudaMemcpyAsync(&s->amg_pin[0], C.rowptr + nc, sizeof(int), cudaMemcpyDeviceToHost, st));
-    VAG_CUDA(cudaMemcpyAsync(&s->amg_pin[1], s->status, sizeof(int), cudaMemcpyDeviceToHost, st));
-    VAG_CUDA(cudaMemcpyAsync(C.sys_start.data(), C.d_sys_start, 4 * (ns + 1), cudaMemcpyDeviceToHost, st));
+    int *starts = static_cast<int *>(ctx_stage(s->ctx, 4 * ((size_t)ns + 1)));
+    VAG_CUDA(cudaMemcpyAsync(&pin[0], C.rowptr + nc, sizeof(int), cudaMemcpyDeviceToHost, st));
+    VAG_CUDA(cudaMemcpyAsync(&pin[1], s->status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    VAG_CUDA(cudaMemcpyAsync(starts, C.d_sys_start, 4 * ((size_t)ns + 1), cudaMemcpyDeviceToHost, st));
     VAG_CUDA(cudaStreamSynchronize(st));
-    C.nnz = s->amg_pin[0];
-    const int cst = s->amg_pin[1];
+    C.nnz = pin[0];
+    const int cst = pin[1];
+    C.sys_start.assign(starts, starts + ns + 1);
     if (cst & ST_ROW_OVERFLOW) fail(VAG_EMESH, "AMG: a coarse row couples too many aggregates");
     if (cst & ST_NONPOSITIVE) fail(VAG_EINVAL, "AMG: non-positive coarse diagonal");
     C.col = static_cast<int *>(alloc(4 * (size_t)std::max<int64_t>(C.nnz, 1)));
     C.val = static_cast<double *>(alloc(8 * (size_t)std::max<int64_t>(C.nnz, 1)));
     k_coarse_compact<<<grid_for(nc, TB), TB, 0, st>>>(nc, tcol, tval, C.rowptr, C.col, C.val);
     note_launches(1);
-    VAG_CUDA(cudaFreeAsync(tcol, st));
-    VAG_CUDA(cudaFreeAsync(tval, st));
     trace_mark(st, "level: Galerkin product");
     A.levels.push_back(C);   // invalidates L
   }
@@ -1421,8 +1434,11 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
     }
     if (!A.levels.empty()) A.levels[0].r32 = static_cast<float *>(alloc(4 * (size_t)std::max(A.levels[0].n, 1)));
   }
+  VAG_CUDA(cudaMemcpyAsync(&pin[kDenseStatusPin], dense_status, sizeof(int), cudaMemcpyDeviceToHost, st));
+  A.status_pending = true;   // checked when the caller waits for the solve
   // first nonzero of each system on every coarse level (the tail's layout)
-  for (size_t l = 1; l < A.levels.size(); ++l) {
+  const bool may_tail = f32 && !classical;   // the one-kernel tail walks aggregates
+  for (size_t l = 1; may_tail && l < A.levels.size(); ++l) {
     AmgLevel &L = A.levels[l];
     L.d_nz_start = static_cast<int *>(alloc(4 * ((size_t)ns + 1)));
     k_nz_starts<<<grid_for(ns + 1, TB), TB, 0, st>>>(ns, L.d_sys_start, L.rowptr, L.d_nz_start);
@@ -1430,13 +1446,13 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
     L.nz_start.assign(ns + 1, 0);
     VAG_CUDA(cudaMemcpyAsync(L.nz_start.data(), L.d_nz_start, 4 * ((size_t)ns + 1), cudaMemcpyDeviceToHost, st));
   }
-  VAG_CUDA(cudaStreamSynchronize(st));
+  if (may_tail) VAG_CUDA(cudaStreamSynchronize(st));
   // FP32 hierarchy: first level from which every system's remaining levels
   // fit the tail's shared memory; from there the V-cycle runs in one kernel.
   // (Not for FP64: one SM issues about two FP64 FMAs per clock on GB300, so
   // FP64 work must spread over the whole GPU.)
-  A.tail_start = -1;   // the one-kernel tail walks aggregates: not for classical levels
-  for (size_t l0 = 1; f32 && !classical && l0 < A.levels.size() && A.tail_start < 0; ++l0) {
+  A.tail_start = -1;
+  for (size_t l0 = 1; may_tail && l0 < A.levels.size() && A.tail_start < 0; ++l0) {
     if ((int)(A.levels.size() - l0) > kTailLevels) continue;
     size_t need[2] = {0, 0};
     for (int g = 0; g < ns; ++g) {
@@ -1483,6 +1499,13 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
     }
   }
   A.built = true;
+}
+
+void amg_check_status(System *s) {
+  if (!s->amg.status_pending) return;
+  s->amg.status_pending = false;
+  if (ctx_pin(s->ctx)[kDenseStatusPin] & ST_NONPOSITIVE)
+    fail(VAG_EINVAL, "AMG: a terminal block is not positive definite");
 }
 
 // Level arrays of one precision.

@@ -114,8 +114,9 @@ __global__ void k_rs_init(int n, const int *__restrict__ rowptr, const int *__re
 // undecided strong neighbours become coarse
 __global__ void k_rs_pmis_c(int n, const int *__restrict__ rowptr, const int *__restrict__ col,
                             const uint8_t *__restrict__ sflag, const unsigned long long *__restrict__ key,
-                            const int8_t *__restrict__ st_in, int8_t *__restrict__ st_out) {
+                            const int8_t *__restrict__ st_in, int8_t *__restrict__ st_out, int *undecided) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *undecided = 0;   // counted by the round's second half
   if (i >= n) return;
   const int8_t s = st_in[i];
   if (s != 0) {
@@ -504,41 +505,37 @@ void rs_coarsen(System *s, AmgLevel &L, AmgLevel &C, const std::function<void *(
   note_launches(2);
   VAG_CHECK_LAUNCH();
   trace_mark(st, "  classical: strength + measure");
-  // PMIS rounds (two kernels each, states ping-pong), polled every 4 rounds
-  int *und_host = s->n_done_host;   // pinned int
-  bool finished = false;
-  for (int r = 0; r < kMaxRounds; ++r) {
-    VAG_CUDA(cudaMemsetAsync(undecided, 0, sizeof(int), st));
-    k_rs_pmis_c<<<g, TB, 0, st>>>(n, L.rowptr, L.col, sflag, key, sa, sb);
-    k_rs_pmis_f<<<g, TB, 0, st>>>(n, L.rowptr, L.col, sflag, sb, sa, undecided);
-    note_launches(2);
-    if ((r & 3) != 3) continue;
-    VAG_CUDA(cudaMemcpyAsync(und_host, undecided, sizeof(int), cudaMemcpyDeviceToHost, st));
-    VAG_CUDA(cudaStreamSynchronize(st));
-    if (*und_host == 0) {
-      finished = true;
-      break;
-    }
-  }
-  if (!finished) fail(VAG_ECUDA, "AMG: the PMIS splitting did not finish");
-  trace_mark(st, "  classical: PMIS rounds");
+  // PMIS rounds (two kernels each, states ping-pong).  The second pass, P's
+  // row counts and their scans follow without a wait; one read-back then
+  // brings the undecided rows, the coarse count and P's nonzeros (R = P^T has
+  // as many), and rows still undecided take four more rounds and the same
+  // again (a round after the last decision changes nothing).
+  int *pin = ctx_pin(s->ctx);
   int *cflag = static_cast<int *>(tmp(4 * (size_t)std::max(n, 1)));
   int *cidx = static_cast<int *>(tmp(4 * ((size_t)n + 1)));
-  k_rs_second_pass<<<g, TB, 0, st>>>(n, L.rowptr, L.col, L.val, maxneg, sa, sb, cflag);
-  note_launches(1);
-  scan_exclusive(cflag, cidx, n, st, false);
-  const int8_t *state = sb;
-  // P: row counts, then one read-back of the coarse count and of P's
-  // nonzeros (R = P^T has as many)
   int *pcnt = static_cast<int *>(tmp(4 * ((size_t)n + 1)));
   L.prow = static_cast<int *>(alloc(4 * ((size_t)n + 1)));
-  k_rs_p_count<<<g, TB, 0, st>>>(n, L.rowptr, L.col, L.val, maxneg, state, pcnt);
-  note_launches(1);
-  scan_exclusive(pcnt, L.prow, n, st, false);
-  int *pin = s->amg_pin;   // pinned
-  VAG_CUDA(cudaMemcpyAsync(&pin[0], cidx + n, sizeof(int), cudaMemcpyDeviceToHost, st));
-  VAG_CUDA(cudaMemcpyAsync(&pin[1], L.prow + n, sizeof(int), cudaMemcpyDeviceToHost, st));
-  VAG_CUDA(cudaStreamSynchronize(st));
+  const int8_t *state = sb;
+  bool finished = false;
+  for (int r = 0, next = n > 2000 ? 8 : 4; r < kMaxRounds && !finished; next += 4) {
+    for (; r < next; ++r) {
+      k_rs_pmis_c<<<g, TB, 0, st>>>(n, L.rowptr, L.col, sflag, key, sa, sb, undecided);
+      k_rs_pmis_f<<<g, TB, 0, st>>>(n, L.rowptr, L.col, sflag, sb, sa, undecided);
+      note_launches(2);
+    }
+    trace_mark(st, "  classical: PMIS rounds");
+    k_rs_second_pass<<<g, TB, 0, st>>>(n, L.rowptr, L.col, L.val, maxneg, sa, sb, cflag);
+    scan_exclusive(s->ctx, cflag, cidx, n, false);
+    k_rs_p_count<<<g, TB, 0, st>>>(n, L.rowptr, L.col, L.val, maxneg, state, pcnt);
+    scan_exclusive(s->ctx, pcnt, L.prow, n, false);
+    note_launches(2);
+    VAG_CUDA(cudaMemcpyAsync(&pin[0], cidx + n, sizeof(int), cudaMemcpyDeviceToHost, st));
+    VAG_CUDA(cudaMemcpyAsync(&pin[1], L.prow + n, sizeof(int), cudaMemcpyDeviceToHost, st));
+    VAG_CUDA(cudaMemcpyAsync(&pin[2], undecided, sizeof(int), cudaMemcpyDeviceToHost, st));
+    VAG_CUDA(cudaStreamSynchronize(st));
+    finished = pin[2] == 0;
+  }
+  if (!finished) fail(VAG_ECUDA, "AMG: the PMIS splitting did not finish");
   const int nc = pin[0];
   L.p_nnz = pin[1];
   L.pcol = static_cast<int *>(alloc(4 * (size_t)std::max<int64_t>(L.p_nnz, 1)));
@@ -554,7 +551,7 @@ void rs_coarsen(System *s, AmgLevel &L, AmgLevel &C, const std::function<void *(
   VAG_CUDA(cudaMemsetAsync(cursor, 0, 4 * ((size_t)nc + 1), st));
   k_rs_r_count<<<g, TB, 0, st>>>(n, L.prow, L.pcol, rcnt);
   note_launches(1);
-  scan_exclusive(rcnt, L.rrow, nc, st, false);
+  scan_exclusive(s->ctx, rcnt, L.rrow, nc, false);
   L.r_nnz = L.p_nnz;
   L.rcol = static_cast<int *>(alloc(4 * (size_t)std::max<int64_t>(L.r_nnz, 1)));
   L.rval = static_cast<double *>(alloc(8 * (size_t)std::max<int64_t>(L.r_nnz, 1)));
@@ -578,10 +575,18 @@ void rs_coarsen(System *s, AmgLevel &L, AmgLevel &C, const std::function<void *(
                                                                L.prow, L.pcol, L.pval, cc, tcol, tval, C.dinv,
                                                                s->status);
   note_launches(1);
-  scan_exclusive(cc, C.rowptr, nc, st, false);
+  scan_exclusive(s->ctx, cc, C.rowptr, nc, false);
+  C.d_sys_start = static_cast<int *>(alloc(4 * ((size_t)ns + 1)));
+  k_rs_coarse_starts<<<grid_for(ns + 1, TB), TB, 0, st>>>(ns, L.d_sys_start, cidx, C.d_sys_start);
+  note_launches(1);
+  VAG_CHECK_LAUNCH();
+  // one wait for the coarse nonzeros, the status and the row starts
+  int *starts = static_cast<int *>(ctx_stage(s->ctx, 4 * ((size_t)ns + 1)));
   VAG_CUDA(cudaMemcpyAsync(&pin[0], C.rowptr + nc, sizeof(int), cudaMemcpyDeviceToHost, st));
   VAG_CUDA(cudaMemcpyAsync(&pin[1], s->status, sizeof(int), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaMemcpyAsync(starts, C.d_sys_start, 4 * ((size_t)ns + 1), cudaMemcpyDeviceToHost, st));
   VAG_CUDA(cudaStreamSynchronize(st));
+  C.sys_start.assign(starts, starts + ns + 1);
   C.nnz = pin[0];
   {
     const int stv = pin[1];
@@ -595,15 +600,7 @@ void rs_coarsen(System *s, AmgLevel &L, AmgLevel &C, const std::function<void *(
   k_rs_compact<kRapCap><<<grid_for(nc, TB), TB, 0, st>>>(nc, tcol, tval, C.rowptr, C.col, C.val);
   note_launches(1);
   trace_mark(st, "  classical: Galerkin R A P");
-  C.d_sys_start = static_cast<int *>(alloc(4 * ((size_t)ns + 1)));
-  k_rs_coarse_starts<<<grid_for(ns + 1, TB), TB, 0, st>>>(ns, L.d_sys_start, cidx, C.d_sys_start);
-  note_launches(1);
   VAG_CHECK_LAUNCH();
-  C.sys_start.assign(ns + 1, 0);
-  VAG_CUDA(cudaMemcpyAsync(C.sys_start.data(), C.d_sys_start, 4 * ((size_t)ns + 1), cudaMemcpyDeviceToHost, st));
-  const int stv = read_status(s);   // synchronises
-  if (stv & ST_BAD_INDEX) fail(VAG_ECUDA, "AMG: internal sparse-product count mismatch");
-  if (stv & ST_NONPOSITIVE) fail(VAG_EINVAL, "AMG: non-positive coarse diagonal");
 }
 
 }  // namespace vag

@@ -117,22 +117,21 @@ void upload_wells(System *s, const WellsHost &w) {
     s->Fw = sys_alloc<double>(s, n);
     s->perf_cap = n;
   }
+  s->n_perf = n;
+  if (!n) return;
   if (!s->ff_perf) s->ff_perf = sys_alloc<int>(s, s->nf > 0 ? s->nf : 1);
   cudaStream_t st = s->ctx->stream;
-  if (n) {
-    VAG_CUDA(cudaMemsetAsync(s->Fw, 0, sizeof(double) * n, st));   // no well rates before a solve
-    VAG_CUDA(cudaMemcpyAsync(s->well_ff, w.ff.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
-    VAG_CUDA(cudaMemcpyAsync(s->well_wi, w.wi.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
-    VAG_CUDA(cudaMemcpyAsync(s->well_pw, w.pw.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
-    VAG_CUDA(cudaMemcpyAsync(s->well_q, w.q.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
-    VAG_CUDA(cudaMemcpyAsync(s->well_cin, w.cin.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
-  }
+  VAG_CUDA(cudaMemsetAsync(s->Fw, 0, sizeof(double) * n, st));   // no well rates before a solve
+  VAG_CUDA(cudaMemcpyAsync(s->well_ff, w.ff.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
+  VAG_CUDA(cudaMemcpyAsync(s->well_wi, w.wi.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
+  VAG_CUDA(cudaMemcpyAsync(s->well_pw, w.pw.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
+  VAG_CUDA(cudaMemcpyAsync(s->well_q, w.q.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
+  VAG_CUDA(cudaMemcpyAsync(s->well_cin, w.cin.data(), sizeof(double) * n, cudaMemcpyHostToDevice, st));
   // fracture face -> perforation (or -1), for the transport map
   std::vector<int> fp((size_t)(s->nf > 0 ? s->nf : 1), -1);
   for (int i = 0; i < n; ++i) fp[w.ff[i]] = i;
   VAG_CUDA(cudaMemcpyAsync(s->ff_perf, fp.data(), sizeof(int) * fp.size(), cudaMemcpyHostToDevice, st));
   VAG_CUDA(cudaStreamSynchronize(st));   // the host vectors go out of scope
-  s->n_perf = n;
 }
 
 // Shapes of a general mesh: keep the per-cell array only when some cell is
@@ -149,7 +148,8 @@ void copy_out(const System *s, T *dst, const T *src, size_t n, int mem) {
 
 void use_device(Ctx *c) { VAG_CUDA(cudaSetDevice(c->device)); }
 
-// Segment starts of a batch (host vectors already filled) copied to the device.
+// Segment starts of a batch (host vectors already filled) copied to the device
+// (the vectors live as long as the system: no wait).
 void upload_segments(System *s) {
   Segments &g = s->seg;
   const int n1 = g.n_sys + 1;
@@ -157,7 +157,6 @@ void upload_segments(System *s) {
   g.d_ff_start = upload(s, g.ff_start.data(), n1, VAG_MEM_HOST, "ff_start");
   g.d_cell_start = upload(s, g.cell_start.data(), n1, VAG_MEM_HOST, "cell_start");
   g.d_row_start = sys_alloc<int>(s, n1);
-  VAG_CUDA(cudaStreamSynchronize(s->ctx->stream));
 }
 
 __global__ void k_add_offset(int *a, int64_t n, int off) {
@@ -172,6 +171,8 @@ void free_ctx(vag_ctx *ctx) {
     cudaStreamDestroy(ctx->c.own_stream);
   }
   if (ctx->c.pool) cudaMemPoolDestroy(ctx->c.pool);
+  if (ctx->c.pin) cudaFreeHost(ctx->c.pin);
+  if (ctx->c.stage) cudaFreeHost(ctx->c.stage);
   delete ctx;
 }
 
@@ -186,11 +187,9 @@ void destroy_system(vag_system *sys) {
     loop_destroy(*g);
   if (s->step_graph) cudaGraphExecDestroy(s->step_graph);
   amg_free(s);
-  if (s->ks_host) cudaFreeHost(s->ks_host);
-  if (s->n_done_host) cudaFreeHost(s->n_done_host);
-  if (s->amg_pin) cudaFreeHost(s->amg_pin);
   if (s->ev0) cudaEventDestroy(s->ev0);
   if (s->ev1) cudaEventDestroy(s->ev1);
+  if (s->ev2) cudaEventDestroy(s->ev2);
   sys_free_all(s);
   const bool counted = s->counted;
   delete sys;
@@ -299,6 +298,7 @@ vag_status vag_assemble(vag_ctx *ctx, const vag_mesh *mesh, const vag_props *pro
     s->mu = props->mu;
     VAG_CUDA(cudaEventCreate(&s->ev0));
     VAG_CUDA(cudaEventCreate(&s->ev1));
+    VAG_CUDA(cudaEventCreate(&s->ev2));
     trace_mark(s->ctx->stream, "start");
     s->status = sys_alloc<int>(s, 4);
     s->xyz = upload(s, mesh->xyz, 3 * (size_t)s->nv, mem, "xyz");
@@ -333,10 +333,10 @@ vag_status vag_assemble(vag_ctx *ctx, const vag_mesh *mesh, const vag_props *pro
     g.dir_start = {0, s->nd};
     upload_segments(s);
     trace_mark(s->ctx->stream, "upload");
-    symbolic_phase(s);
+    const int64_t sell_total = symbolic_phase(s);
     trace_mark(s->ctx->stream, "symbolic phase");
     build_tiles(s);
-    build_sell(s);
+    build_sell(s, sell_total);
     trace_mark(s->ctx->stream, "row tiles + SELL structure");
     numeric_phase(s);
     trace_mark(s->ctx->stream, "numeric phase");
@@ -381,6 +381,7 @@ vag_status vag_assemble_batch(vag_ctx *ctx, int32_t n_sys, const vag_mesh *meshe
     s->mu = props[0].mu;
     VAG_CUDA(cudaEventCreate(&s->ev0));
     VAG_CUDA(cudaEventCreate(&s->ev1));
+    VAG_CUDA(cudaEventCreate(&s->ev2));
     s->status = sys_alloc<int>(s, 4);
     Segments &g = s->seg;
     g.n_sys = n_sys;
@@ -448,9 +449,9 @@ vag_status vag_assemble_batch(vag_ctx *ctx, int32_t n_sys, const vag_mesh *meshe
     set_shapes(s, shape, mask, tri);
     upload_wells(s, wells);
     upload_segments(s);
-    symbolic_phase(s);
+    const int64_t sell_total = symbolic_phase(s);
     build_tiles(s);
-    build_sell(s);
+    build_sell(s, sell_total);
     numeric_phase(s);
   });
   if (st != VAG_OK) {
@@ -645,17 +646,14 @@ vag_status vag_spmv(vag_system *sys, const double *x, double *y, int mem) {
       spmv_f64(s, x, y);   // stream-ordered: no host synchronisation
       return;
     } else {
-      double *dx, *dy;
       const size_t n = s->n_rows;
-      VAG_CUDA(cudaMallocAsync(&dx, sizeof(double) * n, st));
-      VAG_CUDA(cudaMallocAsync(&dy, sizeof(double) * n, st));
+      Scratch scratch(s->ctx);
+      double *dx = scratch.get<double>(n), *dy = scratch.get<double>(n);
       VAG_CUDA(cudaMemcpyAsync(dx, x, sizeof(double) * n, cudaMemcpyHostToDevice, st));
       spmv_f64(s, dx, dy);
       VAG_CUDA(cudaMemcpyAsync(y, dy, sizeof(double) * n, cudaMemcpyDeviceToHost, st));
-      VAG_CUDA(cudaFreeAsync(dx, st));
-      VAG_CUDA(cudaFreeAsync(dy, st));
+      VAG_CUDA(cudaStreamSynchronize(st));
     }
-    VAG_CUDA(cudaStreamSynchronize(st));
   });
 }
 
@@ -676,29 +674,20 @@ vag_status vag_transport(vag_system *sys, const vag_transport_opts *o, double *c
     cudaStream_t st = s->ctx->stream;
     trace_mark(st, "start");
     const size_t n = s->n_cv;
-    // stage porosities, cbar and c
     if (!o->phi_m || (s->nf && !o->phi_f) || (s->nd && !o->cbar)) fail(VAG_EINVAL, "null porosity or cbar");
-    double *stage;
-    const size_t tot = (size_t)s->nc + s->nf + s->nd + (o->mem == VAG_MEM_HOST ? n : 0);
-    VAG_CUDA(cudaMallocAsync(&stage, sizeof(double) * (tot ? tot : 1), st));
-    double *pm = stage, *pf = stage + s->nc, *cb = pf + s->nf;
-    VAG_CUDA(cudaMemcpyAsync(pm, o->phi_m, sizeof(double) * s->nc, to_dev(o->mem), st));
-    if (s->nf) VAG_CUDA(cudaMemcpyAsync(pf, o->phi_f, sizeof(double) * s->nf, to_dev(o->mem), st));
-    VAG_CUDA(cudaMemcpyAsync(cb, o->cbar, sizeof(double) * s->nd, to_dev(o->mem), st));
-    double *cdev = c_inout;
-    if (o->mem == VAG_MEM_HOST) {
-      cdev = cb + s->nd;
+    if (o->mem == VAG_MEM_DEVICE) {   // the caller's arrays, read and written in stream order
+      transport_run(s, o, c_inout, inf, o->phi_m, o->phi_f, o->cbar);
+    } else {
+      Scratch scratch(s->ctx);
+      double *pm = scratch.get<double>((size_t)s->nc + s->nf + s->nd + n), *pf = pm + s->nc, *cb = pf + s->nf,
+             *cdev = cb + s->nd;
+      VAG_CUDA(cudaMemcpyAsync(pm, o->phi_m, sizeof(double) * s->nc, cudaMemcpyHostToDevice, st));
+      if (s->nf) VAG_CUDA(cudaMemcpyAsync(pf, o->phi_f, sizeof(double) * s->nf, cudaMemcpyHostToDevice, st));
+      if (s->nd) VAG_CUDA(cudaMemcpyAsync(cb, o->cbar, sizeof(double) * s->nd, cudaMemcpyHostToDevice, st));
       VAG_CUDA(cudaMemcpyAsync(cdev, c_inout, sizeof(double) * n, cudaMemcpyHostToDevice, st));
-    }
-    try {
       transport_run(s, o, cdev, inf, pm, pf, cb);
-    } catch (...) {
-      cudaFreeAsync(stage, st);
-      throw;
-    }
-    if (o->mem == VAG_MEM_HOST)
       VAG_CUDA(cudaMemcpyAsync(c_inout, cdev, sizeof(double) * n, cudaMemcpyDeviceToHost, st));
-    VAG_CUDA(cudaFreeAsync(stage, st));
+    }
     trace_mark(st, "copy out");
     VAG_CUDA(cudaStreamSynchronize(st));
     trace_report("vag_transport");

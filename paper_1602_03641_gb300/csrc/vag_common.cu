@@ -115,6 +115,23 @@ void ctx_free(Ctx *c, void *p) {
   else cudaFree(p);
 }
 
+int *ctx_pin(Ctx *c) {
+  if (!c->pin) VAG_CUDA(cudaMallocHost(&c->pin, kPinWords * sizeof(int)));
+  return c->pin;
+}
+
+void *ctx_stage(Ctx *c, size_t bytes) {
+  if (bytes > c->stage_bytes) {
+    if (c->stage) VAG_CUDA(cudaFreeHost(c->stage));
+    c->stage = nullptr;
+    c->stage_bytes = 0;
+    bytes = std::max<size_t>(2 * bytes, 16384);
+    VAG_CUDA(cudaMallocHost(&c->stage, bytes));
+    c->stage_bytes = bytes;
+  }
+  return c->stage;
+}
+
 void *sys_alloc_bytes(System *s, size_t bytes) {
   Ctx *c = s->ctx;
   bytes = (std::max<size_t>(bytes, 1) + 255) & ~size_t(255);   // a zero-size array still gets a valid pointer
@@ -154,18 +171,25 @@ int grid_for(int64_t n, int block) {
 }
 
 int read_status(System *s) {
-  int st = 0;
-  VAG_CUDA(cudaMemcpyAsync(&st, s->status, sizeof(int), cudaMemcpyDeviceToHost, s->ctx->stream));
+  int *pin = ctx_pin(s->ctx);
+  VAG_CUDA(cudaMemcpyAsync(pin, s->status, sizeof(int), cudaMemcpyDeviceToHost, s->ctx->stream));
   VAG_CUDA(cudaStreamSynchronize(s->ctx->stream));
-  return st;
+  return *pin;
 }
 
 // ------------------------------------------------------------------ scan ----
+// Tiles of 4096 values: one kernel sums the tiles, a second one scans them,
+// each block first adding the sums of the tiles before its own (a few
+// thousand values from L2 even for 10^7 inputs).  Two launches whatever the
+// length, one up to 4096 values; the scans of the setup phases are short and
+// many, so that launches are what they cost (tiles of 1024 with a recursive
+// scan of their sums took two to seven).
 namespace {
 constexpr int kScanThreads = 256;
-constexpr int kScanItems = 4;
+constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanThreads * kScanItems;
 
+// exclusive prefix of v over the block's threads; *total in every thread
 __device__ __forceinline__ int block_exclusive_sum(int v, int *total) {
   __shared__ int warp_tot[kScanThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -175,94 +199,74 @@ __device__ __forceinline__ int block_exclusive_sum(int v, int *total) {
     int t = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += t;
   }
+  __syncthreads();   // warp_tot may still be read from a previous call
   if (lane == 31) warp_tot[warp] = incl;
   __syncthreads();
-  if (warp == 0) {
-    int w = lane < kScanThreads / 32 ? warp_tot[lane] : 0;
-    int wi = w;
+  int before = 0, sum = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int t = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += t;
-    }
-    if (lane < kScanThreads / 32) warp_tot[lane] = wi - w;
-    if (lane == kScanThreads / 32 - 1) *total = wi;
+  for (int w = 0; w < kScanThreads / 32; ++w) {
+    if (w < warp) before += warp_tot[w];
+    sum += warp_tot[w];
   }
-  __syncthreads();
-  return incl - v + warp_tot[warp];
+  *total = sum;
+  return incl - v + before;
 }
 
-__global__ void scan_tiles(const int *__restrict__ in, int *__restrict__ out, int *__restrict__ tile_sums,
-                           int n) {
-  __shared__ int tot;
+__global__ void __launch_bounds__(kScanThreads) scan_sums(const int *__restrict__ in, int *__restrict__ sums, int n) {
+  const int64_t base = (int64_t)blockIdx.x * kScanTile;
+  int v = 0;
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i) {
+    const int64_t k = base + i * kScanThreads + threadIdx.x;
+    v += k < n ? in[k] : 0;
+  }
+  int tot;
+  block_exclusive_sum(v, &tot);
+  if (threadIdx.x == 0) sums[blockIdx.x] = tot;
+}
+
+__global__ void __launch_bounds__(kScanThreads) scan_write(const int *__restrict__ in, const int *__restrict__ sums,
+                                                           int *__restrict__ out, int n) {
+  int before = 0;
+  for (int b = threadIdx.x; b < (int)blockIdx.x; b += kScanThreads) before += sums[b];
+  int offset, tot;
+  block_exclusive_sum(before, &offset);
   const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
   int v[kScanItems];
   int sum = 0;
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i) {
-    int64_t idx = base + i;
-    v[i] = idx < n ? in[idx] : 0;
+    v[i] = base + i < n ? in[base + i] : 0;
     sum += v[i];
   }
-  int off = block_exclusive_sum(sum, &tot);
+  int run = offset + block_exclusive_sum(sum, &tot);
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i) {
-    int64_t idx = base + i;
-    if (idx < n) out[idx] = off;
-    off += v[i];
+    if (base + i < n) out[base + i] = run;
+    run += v[i];
   }
-  if (threadIdx.x == 0) tile_sums[blockIdx.x] = tot;
-}
-
-__global__ void add_tile_offsets(int *__restrict__ out, const int *__restrict__ offs, int n) {
-  const int64_t base = (int64_t)blockIdx.x * kScanTile;
-  const int add = offs[blockIdx.x];
-  for (int i = threadIdx.x; i < kScanTile; i += blockDim.x) {
-    int64_t idx = base + i;
-    if (idx < n) out[idx] += add;
-  }
-}
-
-__global__ void write_total(int *out, int n, const int *tile_sums_scanned, int ntiles,
-                            const int *tile_sums) {
-  out[n] = tile_sums_scanned[ntiles - 1] + tile_sums[ntiles - 1];
-}
-
-void scan_rec(const int *in, int *out, int n, cudaStream_t st) {
-  // out has room for n+1 entries; writes exclusive prefix and out[n] = total.
-  int ntiles = (n + kScanTile - 1) / kScanTile;
-  if (ntiles < 1) ntiles = 1;
-  int *sums = nullptr;
-  VAG_CUDA(cudaMallocAsync(&sums, sizeof(int) * (2 * ntiles + 1), st));
-  int *sums_scan = sums + ntiles;
-  scan_tiles<<<ntiles, kScanThreads, 0, st>>>(in, out, sums, n);
-  VAG_CHECK_LAUNCH();
-  note_launches(2);   // scan_tiles + write_total
-  if (ntiles > 1) {
-    scan_rec(sums, sums_scan, ntiles, st);
-    add_tile_offsets<<<ntiles, kScanThreads, 0, st>>>(out, sums_scan, n);
-    VAG_CHECK_LAUNCH();
-    note_launches(1);
-  } else {
-    VAG_CUDA(cudaMemsetAsync(sums_scan, 0, sizeof(int), st));
-  }
-  write_total<<<1, 1, 0, st>>>(out, n, sums_scan, ntiles, sums);
-  VAG_CHECK_LAUNCH();
-  VAG_CUDA(cudaFreeAsync(sums, st));
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = offset + tot;
 }
 }  // namespace
 
-int scan_exclusive(const int *in, int *out, int n, cudaStream_t st, bool want_total) {
+int scan_exclusive(Ctx *c, const int *in, int *out, int n, bool want_total) {
+  cudaStream_t st = c->stream;
   if (n == 0) {
     VAG_CUDA(cudaMemsetAsync(out, 0, sizeof(int), st));
     return 0;
   }
-  scan_rec(in, out, n, st);
+  const int ntiles = (int)(((int64_t)n + kScanTile - 1) / kScanTile);
+  Scratch scratch(c);
+  int *sums = ntiles > 1 ? scratch.get<int>(ntiles) : nullptr;
+  if (ntiles > 1) scan_sums<<<ntiles, kScanThreads, 0, st>>>(in, sums, n);
+  scan_write<<<ntiles, kScanThreads, 0, st>>>(in, sums, out, n);
+  VAG_CHECK_LAUNCH();
+  note_launches(ntiles > 1 ? 2 : 1);
   if (!want_total) return -1;
-  int total = 0;
-  VAG_CUDA(cudaMemcpyAsync(&total, out + n, sizeof(int), cudaMemcpyDeviceToHost, st));
+  int *pin = ctx_pin(c);
+  VAG_CUDA(cudaMemcpyAsync(pin, out + n, sizeof(int), cudaMemcpyDeviceToHost, st));
   VAG_CUDA(cudaStreamSynchronize(st));
-  return total;
+  return *pin;
 }
 
 }  // namespace vag

@@ -296,14 +296,11 @@ void gmres_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   if (!s->kz) s->kz = sys_alloc<double>(s, s->n_rows);
   double *V = s->gm_V, *w = s->gm_w, *z = s->kz;
   GmState *gs = reinterpret_cast<GmState *>(s->gm_state);
-  float setup_ms = 0.f;
   VAG_CUDA(cudaEventRecord(s->ev0, st));
   if (amg || cheb) {
     if (amg) amg_setup(s, o->precision != VAG_FP64, o->precision == VAG_MIXED_F16, o->precond == VAG_PC_AMG_RS);
     else cheb_setup(s);
-    VAG_CUDA(cudaEventRecord(s->ev1, st));
-    VAG_CUDA(cudaEventSynchronize(s->ev1));
-    cudaEventElapsedTime(&setup_ms, s->ev0, s->ev1);
+    VAG_CUDA(cudaEventRecord(s->ev2, st));
   }
   // z = M v; in_iter: systems already done are skipped where the
   // preconditioner allows it (the AMG V-cycle runs for every system)
@@ -354,17 +351,19 @@ void gmres_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   }
   VAG_CUDA(cudaMemsetAsync(s->kx, 0, sizeof(double) * s->n_rows, st));
   restart(1);
+  int *pin = ctx_pin(s->ctx);
+  auto all_done = [&]() {
+    VAG_CUDA(cudaMemcpyAsync(pin, s->n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
+    VAG_CUDA(cudaStreamSynchronize(st));
+    return *pin >= ns;
+  };
   const int max_cycles = o->maxit + 2;   // an active system makes at least one step per cycle
   for (int cyc = 0; cyc < max_cycles; ++cyc) {
-    VAG_CUDA(cudaMemcpyAsync(s->n_done_host, s->n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
-    VAG_CUDA(cudaStreamSynchronize(st));
-    if (*s->n_done_host >= ns) break;
+    if (all_done()) break;
     for (int c = 0; c < nchunks; ++c) {
       VAG_CUDA(cudaGraphLaunch(chunks[c], st));
       note_launches(chunk_nodes[c]);
-      VAG_CUDA(cudaMemcpyAsync(s->n_done_host, s->n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
-      VAG_CUDA(cudaStreamSynchronize(st));
-      if (*s->n_done_host >= ns) break;
+      if (all_done()) break;
     }
     // x += M V_k y for every system that made steps in this cycle
     k_gm_solve<<<(ns + 127) / 128, 128, 0, st>>>(ns, gs);
@@ -380,8 +379,7 @@ void gmres_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   // the true residual decides the status
   true_residual2(s, st);
   finish_solve(s, info, false);
-  info->ms_setup = setup_ms;
-  info->ms_solve -= setup_ms;
+  if (amg || cheb) split_setup_time(s, info);
 }
 
 }  // namespace vag

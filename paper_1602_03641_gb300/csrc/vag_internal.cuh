@@ -66,6 +66,11 @@ struct Ctx {
   cudaStream_t own_stream = nullptr;
   cudaStream_t stream = nullptr;
   cudaMemPool_t pool = nullptr;   // stream-ordered pool for every device buffer of the context's systems
+  // pinned read-back words (see ctx_pin) and a pinned staging buffer that
+  // grows (see ctx_stage), both released with the context
+  int *pin = nullptr;
+  void *stage = nullptr;
+  size_t stage_bytes = 0;
   std::string last_error;
   // autotuned loads in flight of the sliced-ELL row loop, per matrix size
   // class (floor(log2 rows)); see tune_sell
@@ -106,6 +111,7 @@ struct AmgLevel {
   bool any_term = false, all_term = false;
   double *inv = nullptr;           // dense inverses of the terminal blocks
   long long *inv_off = nullptr;    // [n_sys+1] offsets (0-sized for other systems)
+  std::vector<long long> inv_off_h;
   long long n_inv = 0;             // entries of inv
   int nc = 0;
   int *mptr = nullptr, *mem = nullptr;   // members of each aggregate, sorted
@@ -134,6 +140,7 @@ struct Amg {
   std::vector<void *> allocs;
   size_t bytes = 0;
   bool built = false;
+  bool status_pending = false;     // the terminal blocks' status is on its way to the pinned words
   bool f32 = false;                // V-cycle in FP32
   bool classical = false;          // classical (Ruge-Stueben-type) levels instead of aggregation
   int tail_start = -1;             // first level run by the one-kernel tail
@@ -152,7 +159,7 @@ struct Amg {
 // body while its condition is non-zero (it starts at 1 with every launch; a
 // kernel of the body sets it to 0, see loop_end_check).  Against graphs of 8
 // or 16 iterations that the host polled, no iteration and no V-cycle runs
-// past the last one (56 of 45 ran in the 128^3 mixed solve) and one
+// past the last one (56 ran where 45 were needed in the 128^3 mixed solve) and one
 // iteration is captured instead of a chunk: 128^3 run 148.7 -> 137.8 ms, 96^3
 // FP64 CG with the FP32 V-cycle 46.9 -> 40.1 ms, batch of 32 49.3 -> 43.9 ms,
 // the same bits.
@@ -186,7 +193,8 @@ struct Segments {
   std::vector<int> node_start, ff_start, cell_start, dir_start, row_start;   // host, n_sys+1
   int *d_node_start = nullptr, *d_ff_start = nullptr, *d_cell_start = nullptr, *d_row_start = nullptr;
   int n_tiles = 0;
-  std::vector<int> tile_start_h;     // first tile of each system, n_sys+1
+  std::vector<int> tile_start_h;     // first tile and first reduction group of each system, n_sys+1
+  std::vector<int> group_start_h;
   int *tile_sys = nullptr;           // [n_tiles]
   int *tile_row0 = nullptr;          // [n_tiles+1] (row range of tile t: [row0[t], row1[t]))
   int *tile_row1 = nullptr;
@@ -223,7 +231,7 @@ struct System {
   int *well_ff = nullptr;      // [n_perf] fracture-face index (distinct)
   double *well_wi = nullptr, *well_pw = nullptr, *well_q = nullptr, *well_cin = nullptr;   // [n_perf]
   double *Fw = nullptr;        // [n_perf] rate leaving the face into the well
-  int *ff_perf = nullptr;      // [nf] perforation of each fracture face, or -1
+  int *ff_perf = nullptr;      // [nf] perforation of each fracture face, or -1 (set when n_perf > 0)
   int perf_cap = 0;
   int *dir_nodes = nullptr;
   double *dir_vals = nullptr;
@@ -270,10 +278,8 @@ struct System {
   double *partials = nullptr;  // [2 * n_tiles] (Krylov) / [kMaxRedBlocks] (transport)
   unsigned int *counter = nullptr;     // [n_sys + 1] arrival counters
   KrylovScalars *ks = nullptr;         // [n_sys]
-  KrylovScalars *ks_host = nullptr;    // pinned mirror [n_sys]
+  std::vector<KrylovScalars> ks_host;  // their last values read back
   int *n_done = nullptr;               // [2] systems converged, passes over loop bodies (device)
-  int *n_done_host = nullptr;          // pinned mirror [2]
-  int *amg_pin = nullptr;              // pinned, 4 ints: AMG setup read-backs
   Segments seg;
   LoopGraph pcg_loop;          // Krylov iterations: Jacobi, AMG (rebuilt per solve), Chebyshev, BiCGStab
   LoopGraph pcg_loop_amg, pcg_loop_cheb, bicg_loop;
@@ -318,7 +324,7 @@ struct System {
   std::vector<double> dts_host;
 
   // timing events
-  cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;   // ev2: end of a preconditioner's setup
 };
 
 // allocation helpers (budget-checked)
@@ -326,6 +332,36 @@ void *sys_alloc_bytes(System *s, size_t bytes);
 // device allocation from the context's pool (stream-ordered on its stream)
 void *ctx_alloc(Ctx *c, size_t bytes);
 void ctx_free(Ctx *c, void *p);
+// Pinned read-back words of the context (kPinWords ints), allocated with the
+// first use; a caller waits for its own copies into them before it returns.
+constexpr int kPinWords = 64;
+int *ctx_pin(Ctx *c);
+// Pinned staging buffer of at least `bytes` bytes.  Callers wait for the
+// stream before they read it and before they ask for it again.
+void *ctx_stage(Ctx *c, size_t bytes);
+// Temporaries of the context's pool, stream-ordered, released on every path.
+// (The device's default pool hands its memory back to the driver at every
+// synchronisation, and each scratch array then pays for a driver allocation,
+// tens of microseconds apiece: with the context's pool, fewer waits and no
+// pinned allocation per system, a run on 83 000 prisms went from 14.9 to 8.3
+// ms, on 280 000 tetrahedra from 19.8 to 12.4 ms, at 128^3 from 137.8 to
+// 127.9 ms.)
+struct Scratch {
+  Ctx *c;
+  std::vector<void *> p;
+  explicit Scratch(Ctx *ctx) : c(ctx) {}
+  Scratch(const Scratch &) = delete;
+  Scratch &operator=(const Scratch &) = delete;
+  ~Scratch() {
+    for (void *q : p) ctx_free(c, q);
+  }
+  template <class T>
+  T *get(size_t n) {
+    void *q = ctx_alloc(c, (n ? n : 1) * sizeof(T));
+    p.push_back(q);
+    return static_cast<T *>(q);
+  }
+};
 template <class T>
 T *sys_alloc(System *s, size_t n) {
   return static_cast<T *>(sys_alloc_bytes(s, (n ? n : 1) * sizeof(T)));
@@ -408,9 +444,10 @@ __device__ __forceinline__ void loop_system_done(cudaGraphConditionalHandle loop
 }
 #endif
 
-// Exclusive scan of n int32 values: out[0..n] (out[n] = total).  Returns the
-// total (synchronises the stream).
-int scan_exclusive(const int *in, int *out, int n, cudaStream_t st, bool want_total = true);
+// Exclusive scan of n int32 values on the context's stream: out[0..n] (out[n]
+// = total).  Returns the total (synchronises the stream), or -1 at once with
+// want_total = false.
+int scan_exclusive(Ctx *c, const int *in, int *out, int n, bool want_total = true);
 int read_status(System *s);
 int grid_for(int64_t n, int block);
 int num_sms();
@@ -437,7 +474,8 @@ unsigned general_to_cells(Ctx *c, const vag_mesh &m, int mem, int32_t *cell_node
                           int8_t *cell_shape, bool *tri_ff);
 
 // ------------------------------------------------------------- phases -----
-void symbolic_phase(System *s);
+// returns the entries of the sliced-ELL copy (sell_slices)
+int64_t symbolic_phase(System *s);
 void numeric_phase(System *s);
 double time_cell_local(System *s, int reps);   // mean ms of the local-matrix launches of one numeric phase
 void pcg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info);
@@ -468,6 +506,8 @@ bool amg_apply_cg(System *s, const double *r, double *z, cudaStream_t st);
 const float *amg_first_sweep_scale_f32(System *s, float *&t0, float &omega);
 bool amg_apply_f32_cg(System *s, const float *r, float *z, cudaStream_t st, KrylovScalars *ks, int *n_done);
 void amg_free(System *s);
+// after a wait for the stream: fails if a terminal block of the last setup was not positive definite
+void amg_check_status(System *s);
 // Chebyshev preconditioner (FP64): cheb_setup estimates each system's interval
 // from Jacobi-CG Lanczos coefficients and fills the coefficient table;
 // cheb_apply forms z = M r (in_iter: systems already done are skipped;
@@ -497,15 +537,16 @@ void ensure_krylov_buffers(System *s);
 // Krylov result in s->kx and per-system scalars in s->ks: scatter into u,
 // recover the cells, compute the fluxes, fill the aggregate info.
 void finish_solve(System *s, vag_solve_info *info, bool mixed);
+// after finish_solve: the time from ev0 to ev2 moved from ms_solve to ms_setup
+void split_setup_time(System *s, vag_solve_info *info);
 void spmv_f64(System *s, const double *x, double *y);
 void build_tiles(System *s);
-void build_sell(System *s);
+void build_sell(System *s, int64_t total);
 void sell_values(System *s);
 void sell_values_scaled_f32(System *s, const double *scale, float *out);
 void sell_values_f32(System *s, float *out);
 void sell_values_scaled_f16(System *s, const double *scale, __half *out);
-int64_t sell_structure(cudaStream_t st, int n, const int *rowptr, const int *col, int **slice_ptr_out,
-                       int **scol_out, const std::function<void *(size_t)> &alloc);
+void sell_slices(System *s);   // slice_ptr of the eliminated system (no wait; build_sell takes the total)
 void solve_infos(const System *s, vag_solve_info *infos);
 void recover_cells_and_fluxes(System *s);
 void transport_run(System *s, const vag_transport_opts *o, double *c_dev, vag_transport_info *info,

@@ -496,41 +496,61 @@ __global__ void __launch_bounds__(NT) k_bi_pdir(double *__restrict__ p, const do
 // price of small tiles, a longer list of partial sums for the last tile of a
 // system to add, is a few microseconds.)  The tiling depends on the system
 // alone.
-static int tile_rows(int) { return 256; }
+constexpr int kTileRows = 256;
+
+// the tiles of every system's rows, from its first tile (one thread a tile)
+__global__ void k_tiles(int n_tiles, int n_sys, int rows, const int *__restrict__ sys_tile0,
+                        const int *__restrict__ row_start, int *__restrict__ tile_sys, int *__restrict__ row0,
+                        int *__restrict__ row1) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n_tiles) return;
+  int lo = 0, hi = n_sys - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (sys_tile0[mid] <= t) lo = mid; else hi = mid - 1;
+  }
+  const int a = row_start[lo] + rows * (t - sys_tile0[lo]), end = row_start[lo + 1];
+  tile_sys[t] = lo;
+  row0[t] = a;
+  row1[t] = min(a + rows, end);
+}
 
 void build_tiles(System *s) {
   Segments &g = s->seg;
-  std::vector<int> tsys, t0, t1, st(g.n_sys + 1);
+  g.tile_start_h.assign(g.n_sys + 1, 0);
+  g.group_start_h.assign(g.n_sys + 1, 0);
   for (int i = 0; i < g.n_sys; ++i) {
-    st[i] = (int)tsys.size();
-    const int a = g.row_start[i], b = g.row_start[i + 1];
-    const int T = tile_rows(b - a);
-    int r = a;
-    do {   // at least one (possibly empty) tile per system
-      tsys.push_back(i);
-      t0.push_back(r);
-      t1.push_back(std::min(r + T, b));
-      r += T;
-    } while (r < b);
+    const int rows = g.row_start[i + 1] - g.row_start[i];
+    const int tiles = std::max(1, (rows + kTileRows - 1) / kTileRows);   // at least one (possibly empty) tile per system
+    g.tile_start_h[i + 1] = g.tile_start_h[i] + tiles;
+    g.group_start_h[i + 1] = g.group_start_h[i] + (tiles + kSegGroup - 1) / kSegGroup;   // reduction groups
   }
-  st[g.n_sys] = (int)tsys.size();
-  g.n_tiles = (int)tsys.size();
-  g.tile_start_h = st;
-  std::vector<int> gr(g.n_sys + 1, 0);   // reduction groups of each system's tiles
-  for (int i = 0; i < g.n_sys; ++i) gr[i + 1] = gr[i] + (st[i + 1] - st[i] + kSegGroup - 1) / kSegGroup;
-  g.n_groups = gr[g.n_sys];
+  g.n_tiles = g.tile_start_h[g.n_sys];
+  g.n_groups = g.group_start_h[g.n_sys];
   g.sys_grp0 = sys_alloc<int>(s, g.n_sys + 1);
   g.tile_sys = sys_alloc<int>(s, g.n_tiles);
   g.tile_row0 = sys_alloc<int>(s, g.n_tiles);
   g.tile_row1 = sys_alloc<int>(s, g.n_tiles);
   g.sys_tile0 = sys_alloc<int>(s, g.n_sys + 1);
   cudaStream_t str = s->ctx->stream;
-  VAG_CUDA(cudaMemcpyAsync(g.tile_sys, tsys.data(), sizeof(int) * g.n_tiles, cudaMemcpyHostToDevice, str));
-  VAG_CUDA(cudaMemcpyAsync(g.tile_row0, t0.data(), sizeof(int) * g.n_tiles, cudaMemcpyHostToDevice, str));
-  VAG_CUDA(cudaMemcpyAsync(g.tile_row1, t1.data(), sizeof(int) * g.n_tiles, cudaMemcpyHostToDevice, str));
-  VAG_CUDA(cudaMemcpyAsync(g.sys_tile0, st.data(), sizeof(int) * (g.n_sys + 1), cudaMemcpyHostToDevice, str));
-  VAG_CUDA(cudaMemcpyAsync(g.sys_grp0, gr.data(), sizeof(int) * (g.n_sys + 1), cudaMemcpyHostToDevice, str));
-  VAG_CUDA(cudaStreamSynchronize(str));   // host vectors go out of scope
+  // (the host vectors live as long as the system: no wait)
+  VAG_CUDA(cudaMemcpyAsync(g.sys_tile0, g.tile_start_h.data(), sizeof(int) * (g.n_sys + 1), cudaMemcpyHostToDevice,
+                           str));
+  VAG_CUDA(cudaMemcpyAsync(g.sys_grp0, g.group_start_h.data(), sizeof(int) * (g.n_sys + 1), cudaMemcpyHostToDevice,
+                           str));
+  k_tiles<<<grid_for(g.n_tiles, NT), NT, 0, str>>>(g.n_tiles, g.n_sys, kTileRows, g.sys_tile0, g.d_row_start,
+                                                   g.tile_sys, g.tile_row0, g.tile_row1);
+  note_launches(1);
+  VAG_CHECK_LAUNCH();
+}
+
+// The per-system scalars read back into ks_host (waits for the stream).
+static void read_scalars(System *s) {
+  const size_t bytes = sizeof(KrylovScalars) * s->seg.n_sys;
+  KrylovScalars *h = static_cast<KrylovScalars *>(ctx_stage(s->ctx, bytes));
+  VAG_CUDA(cudaMemcpyAsync(h, s->ks, bytes, cudaMemcpyDeviceToHost, s->ctx->stream));
+  VAG_CUDA(cudaStreamSynchronize(s->ctx->stream));
+  s->ks_host.assign(h, h + s->seg.n_sys);
 }
 
 static void launch_spmv_u(System *s, int u, const double *x, double *y, int with_dot, cudaStream_t st) {
@@ -604,8 +624,6 @@ void ensure_krylov_buffers(System *s) {
   s->u = sys_alloc<double>(s, (size_t)s->n_cv);
   VAG_CUDA(cudaMemsetAsync(s->counter, 0, (ns + 1 + s->seg.n_groups) * sizeof(unsigned), s->ctx->stream));
   VAG_CUDA(cudaMemsetAsync(s->u, 0, sizeof(double) * s->n_cv, s->ctx->stream));
-  if (!s->ks_host) VAG_CUDA(cudaMallocHost(&s->ks_host, sizeof(KrylovScalars) * ns));
-  if (!s->n_done_host) VAG_CUDA(cudaMallocHost(&s->n_done_host, 2 * sizeof(int)));
 }
 
 void launch_spmv_plain(System *s, const double *x, double *y, cudaStream_t st) { launch_spmv(s, x, y, 0, st); }
@@ -645,9 +663,10 @@ constexpr int kLoopUnroll = 4;
 // Kernels of the passes over a loop's body so far (System::n_done[1]), for
 // the launch count.  Waits for the loop.
 static void note_loop(System *s, const LoopGraph &g) {
-  VAG_CUDA(cudaMemcpyAsync(s->n_done_host, s->n_done, 2 * sizeof(int), cudaMemcpyDeviceToHost, s->ctx->stream));
+  int *pin = ctx_pin(s->ctx);
+  VAG_CUDA(cudaMemcpyAsync(pin, s->n_done, 2 * sizeof(int), cudaMemcpyDeviceToHost, s->ctx->stream));
   VAG_CUDA(cudaStreamSynchronize(s->ctx->stream));
-  note_launches((unsigned long long)s->n_done_host[1] * g.nodes);
+  note_launches((unsigned long long)pin[1] * g.nodes);
 }
 
 // One iteration of CG with the V-cycle, from r (and its first sweep t0) to
@@ -713,8 +732,7 @@ void jacobi_cg_coefficients(System *s, const double *v, int m, std::vector<doubl
   for (int j = 0; j < m; ++j) {
     pcg_iteration(s, st);
     VAG_CHECK_LAUNCH();
-    VAG_CUDA(cudaMemcpyAsync(s->ks_host, s->ks, sizeof(KrylovScalars) * ns, cudaMemcpyDeviceToHost, st));
-    VAG_CUDA(cudaStreamSynchronize(st));
+    read_scalars(s);
     for (int i = 0; i < ns; ++i) {
       const KrylovScalars &k = s->ks_host[i];
       if (steps[i] != j || k.iter != j + 1 || k.breakdown) continue;
@@ -736,16 +754,13 @@ void pcg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   const int ns = s->seg.n_sys;
   const int nt = s->seg.n_tiles;
   const Tiles tl = tiles_of(s);
-  float setup_ms = 0.f;
   VAG_CUDA(cudaEventRecord(s->ev0, st));
   if (general) {
     if (!s->kz) s->kz = sys_alloc<double>(s, s->n_rows);
     if (amg) amg_setup(s, o->precision != VAG_FP64, o->precision == VAG_MIXED_F16, o->precond == VAG_PC_AMG_RS);
     else cheb_setup(s);
     trace_mark(st, amg ? "AMG setup" : "Chebyshev setup (Lanczos bounds)");
-    VAG_CUDA(cudaEventRecord(s->ev1, st));
-    VAG_CUDA(cudaEventSynchronize(s->ev1));
-    cudaEventElapsedTime(&setup_ms, s->ev0, s->ev1);
+    VAG_CUDA(cudaEventRecord(s->ev2, st));
   }
   // the first step of the preconditioner, formed where r is (the V-cycle's
   // first sweep, the polynomial's first step)
@@ -798,8 +813,7 @@ void pcg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     VAG_CHECK_LAUNCH();
     trace_mark(st, "true residual");
     if (attempt == 3) break;
-    VAG_CUDA(cudaMemcpyAsync(s->ks_host, s->ks, sizeof(KrylovScalars) * ns, cudaMemcpyDeviceToHost, st));
-    VAG_CUDA(cudaStreamSynchronize(st));
+    read_scalars(s);
     bool again = false;
     prev_res2.resize(ns, INFINITY);
     for (int i = 0; i < ns; ++i) {
@@ -811,7 +825,9 @@ void pcg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     }
     if (!again) break;
     // push the stall flags back before the restart kernels read them
-    VAG_CUDA(cudaMemcpyAsync(s->ks, s->ks_host, sizeof(KrylovScalars) * ns, cudaMemcpyHostToDevice, st));
+    KrylovScalars *stage = static_cast<KrylovScalars *>(ctx_stage(s->ctx, sizeof(KrylovScalars) * ns));
+    std::copy(s->ks_host.begin(), s->ks_host.end(), stage);
+    VAG_CUDA(cudaMemcpyAsync(s->ks, stage, sizeof(KrylovScalars) * ns, cudaMemcpyHostToDevice, st));
     VAG_CUDA(cudaMemsetAsync(s->n_done, 0, sizeof(int), st));
     if (general)
       k_restart_m<<<nt, NT, 0, st>>>(s->rhs, s->kq, s->kr, s->kp, tl, s->partials, s->counter, s->ks, s->n_done,
@@ -824,8 +840,7 @@ void pcg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   }
   note_loop(s, loop);
   finish_solve(s, info, false);
-  info->ms_setup = setup_ms;
-  info->ms_solve -= setup_ms;
+  if (amg || cheb) split_setup_time(s, info);
 }
 
 void bicgstab_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
@@ -843,19 +858,14 @@ void bicgstab_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     s->b_t = sys_alloc<double>(s, s->n_rows);
     s->b_ph = sys_alloc<double>(s, s->n_rows);
   }
-  float setup_ms = 0.f;
   VAG_CUDA(cudaEventRecord(s->ev0, st));
   if (amg) {
     if (!s->kz) s->kz = sys_alloc<double>(s, s->n_rows);
     amg_setup(s, o->precision != VAG_FP64, o->precision == VAG_MIXED_F16, o->precond == VAG_PC_AMG_RS);
-    VAG_CUDA(cudaEventRecord(s->ev1, st));
-    VAG_CUDA(cudaEventSynchronize(s->ev1));
-    cudaEventElapsedTime(&setup_ms, s->ev0, s->ev1);
+    VAG_CUDA(cudaEventRecord(s->ev2, st));
   } else if (cheb) {
     cheb_setup(s);
-    VAG_CUDA(cudaEventRecord(s->ev1, st));
-    VAG_CUDA(cudaEventSynchronize(s->ev1));
-    cudaEventElapsedTime(&setup_ms, s->ev0, s->ev1);
+    VAG_CUDA(cudaEventRecord(s->ev2, st));
   }
   auto precond = [&](const double *in, double *out) {
     if (amg) {
@@ -896,8 +906,14 @@ void bicgstab_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   note_launches(1);
   VAG_CHECK_LAUNCH();
   finish_solve(s, info, false);
-  info->ms_setup = setup_ms;
-  info->ms_solve -= setup_ms;
+  if (amg || cheb) split_setup_time(s, info);
+}
+
+void split_setup_time(System *s, vag_solve_info *info) {
+  float ms = 0.f;
+  cudaEventElapsedTime(&ms, s->ev0, s->ev2);
+  info->ms_setup = ms;
+  info->ms_solve -= ms;
 }
 
 static vag_solve_info info_of(const KrylovScalars &k, bool mixed) {
@@ -920,8 +936,8 @@ void finish_solve(System *s, vag_solve_info *info, bool mixed) {
   recover_cells_and_fluxes(s);
   trace_mark(st, "scatter + cell recovery + fluxes");
   VAG_CUDA(cudaEventRecord(s->ev1, st));
-  VAG_CUDA(cudaMemcpyAsync(s->ks_host, s->ks, sizeof(KrylovScalars) * ns, cudaMemcpyDeviceToHost, st));
-  VAG_CUDA(cudaStreamSynchronize(st));
+  read_scalars(s);
+  amg_check_status(s);
   float ms = 0.f;
   cudaEventElapsedTime(&ms, s->ev0, s->ev1);
   // aggregate over the batch: most iterations, worst residual, worst status

@@ -448,12 +448,12 @@ constexpr int kLoopUnroll = 4;
 // kernels of the step's inner loop go to the launch count.
 static bool poll(System *s, int outer, const LoopGraph &inner) {
   cudaStream_t st = s->ctx->stream;
-  VAG_CUDA(cudaMemcpyAsync(&s->n_done_host[0], s->n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
-  if (outer)
-    VAG_CUDA(cudaMemcpyAsync(&s->n_done_host[1], s->mx.n_done_in + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
+  int *pin = ctx_pin(s->ctx);
+  VAG_CUDA(cudaMemcpyAsync(&pin[0], s->n_done, sizeof(int), cudaMemcpyDeviceToHost, st));
+  if (outer) VAG_CUDA(cudaMemcpyAsync(&pin[1], s->mx.n_done_in + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
   VAG_CUDA(cudaStreamSynchronize(st));
-  if (outer) note_launches((unsigned long long)s->n_done_host[1] * inner.nodes);
-  return s->n_done_host[0] >= s->seg.n_sys;
+  if (outer) note_launches((unsigned long long)pin[1] * inner.nodes);
+  return pin[0] >= s->seg.n_sys;
 }
 
 static void ensure_mixed_buffers(System *s) {
@@ -537,10 +537,7 @@ void mixed_amg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     m.dstale = false;
   }
   trace_mark(st, "AMG setup (FP32 hierarchy), difference-form FP32 values");
-  VAG_CUDA(cudaEventRecord(s->ev1, st));
-  VAG_CUDA(cudaEventSynchronize(s->ev1));
-  float setup_ms = 0.f;
-  cudaEventElapsedTime(&setup_ms, s->ev0, s->ev1);
+  VAG_CUDA(cudaEventRecord(s->ev2, st));
   const float *a32 = m.dval32;   // FP32 difference-form values of A, sliced ELL
   auto spmv32 = s->sell_u == 2 ? k_spmv32d<2> : s->sell_u == 8 ? k_spmv32d<8> : k_spmv32d<4>;
   // one inner iteration, from r (and the V-cycle's first sweep) to the next r:
@@ -589,8 +586,7 @@ void mixed_amg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     trace_mark(st, "refinement step");
   }
   finish_solve(s, info, /*mixed=*/true);
-  info->ms_setup = setup_ms;
-  info->ms_solve -= setup_ms;
+  split_setup_time(s, info);
 }
 
 // Mean duration of the inner product q = A p with its p.q reduction, as the

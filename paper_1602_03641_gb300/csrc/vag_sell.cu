@@ -5,8 +5,6 @@
 // (no cross-lane reduction -- on GB300 the FP64 pipe, not HBM, limits a
 // lane-split CSR SpMV).  Entries of a row keep their CSR order, so a row sum
 // is the same sequence of FMAs whatever the slice layout.
-#include <functional>
-
 #include "vag_internal.cuh"
 
 namespace vag {
@@ -69,37 +67,30 @@ __global__ void k_sell_vals(int n, const int *__restrict__ rowptr, const double 
 
 }  // namespace
 
-// Sliced-ELL structure of any CSR matrix (n rows): slice_ptr [n_slices+1]
-// and scol [total]; returns total.  The caller supplies the allocator.
-int64_t sell_structure(cudaStream_t st, int n, const int *rowptr, const int *col, int **slice_ptr_out,
-                       int **scol_out, const std::function<void *(size_t)> &alloc) {
-  const int n_slices = (n + 31) / 32;
-  int *slice_ptr = static_cast<int *>(alloc(sizeof(int) * ((size_t)n_slices + 1)));
-  int *width;
-  VAG_CUDA(cudaMallocAsync(&width, sizeof(int) * ((size_t)n_slices + 1), st));
-  k_slice_width<<<grid_for(n_slices, TB), TB, 0, st>>>(n, n_slices, rowptr, width);
+void sell_slices(System *s) {
+  cudaStream_t st = s->ctx->stream;
+  s->n_slices = (s->n_rows + 31) / 32;
+  s->slice_ptr = sys_alloc<int>(s, (size_t)s->n_slices + 1);
+  Scratch scratch(s->ctx);
+  int *width = scratch.get<int>((size_t)s->n_slices + 1);
+  k_slice_width<<<grid_for(s->n_slices, TB), TB, 0, st>>>(s->n_rows, s->n_slices, s->rowptr, width);
   note_launches(1);
   VAG_CHECK_LAUNCH();
-  const int64_t total = n_slices ? scan_exclusive(width, slice_ptr, n_slices, st) : 0;
-  if (!n_slices) VAG_CUDA(cudaMemsetAsync(slice_ptr, 0, sizeof(int), st));
-  VAG_CUDA(cudaFreeAsync(width, st));
-  int *scol = static_cast<int *>(alloc(sizeof(int) * (size_t)std::max<int64_t>(total, 1)));
+  scan_exclusive(s->ctx, width, s->slice_ptr, s->n_slices, false);
+}
+
+void build_sell(System *s, int64_t total) {
+  cudaStream_t st = s->ctx->stream;
+  const int n = s->n_rows;
+  s->sell_nnz = total;
+  s->scol = sys_alloc<int>(s, (size_t)std::max<int64_t>(total, 1));
+  s->sval = sys_alloc<double>(s, (size_t)std::max<int64_t>(total, 1));
   if (n > 0) {
-    k_sell_cols<<<grid_for(n, TB), TB, 0, st>>>(n, rowptr, col, slice_ptr, scol);
-    k_sell_pad<<<grid_for((int64_t)n_slices * 32, TB), TB, 0, st>>>(n, rowptr, slice_ptr, scol);
+    k_sell_cols<<<grid_for(n, TB), TB, 0, st>>>(n, s->rowptr, s->col, s->slice_ptr, s->scol);
+    k_sell_pad<<<grid_for((int64_t)s->n_slices * 32, TB), TB, 0, st>>>(n, s->rowptr, s->slice_ptr, s->scol);
     note_launches(2);
     VAG_CHECK_LAUNCH();
   }
-  *slice_ptr_out = slice_ptr;
-  *scol_out = scol;
-  return total;
-}
-
-void build_sell(System *s) {
-  s->n_slices = (s->n_rows + 31) / 32;
-  s->sell_nnz = sell_structure(s->ctx->stream, s->n_rows, s->rowptr, s->col, &s->slice_ptr, &s->scol,
-                               [s](size_t bytes) { return sys_alloc_bytes(s, bytes); });
-  s->sval = sys_alloc<double>(s, (size_t)std::max<int64_t>(s->sell_nnz, 1));
 }
 
 void sell_values(System *s) {

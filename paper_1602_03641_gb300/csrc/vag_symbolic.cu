@@ -332,7 +332,7 @@ __global__ void k_row_fill(PatView p, int n_rows, const int *__restrict__ dof_of
 
 }  // namespace
 
-void symbolic_phase(System *s) {
+int64_t symbolic_phase(System *s) {
   cudaStream_t st = s->ctx->stream;
   const int nv = s->nv, nc = s->nc, nf = s->nf, nd = s->nd;
 
@@ -350,18 +350,14 @@ void symbolic_phase(System *s) {
 
   // scratch (stream-ordered, released at the end of the phase)
   const size_t ncnt = (size_t)nv + 1;
-  int *n2c_cnt, *n2f_cnt, *cursor, *ffs, *table, *ff_cnt, *flagv, *scanv;
   uint32_t H = 2;
   while (H < 2u * (uint32_t)(nf > 0 ? nf : 1)) H <<= 1;
   const size_t nflag = std::max<size_t>({(size_t)nc, (size_t)nv + nf, 1}) + 1;
-  VAG_CUDA(cudaMallocAsync(&n2c_cnt, sizeof(int) * ncnt, st));
-  VAG_CUDA(cudaMallocAsync(&n2f_cnt, sizeof(int) * ncnt, st));
-  VAG_CUDA(cudaMallocAsync(&cursor, sizeof(int) * ncnt, st));
-  VAG_CUDA(cudaMallocAsync(&ffs, sizeof(int) * 4 * (size_t)(nf > 0 ? nf : 1), st));
-  VAG_CUDA(cudaMallocAsync(&table, sizeof(int) * H, st));
-  VAG_CUDA(cudaMallocAsync(&ff_cnt, sizeof(int) * (size_t)(nf > 0 ? nf : 1), st));
-  VAG_CUDA(cudaMallocAsync(&flagv, sizeof(int) * nflag, st));
-  VAG_CUDA(cudaMallocAsync(&scanv, sizeof(int) * nflag, st));
+  Scratch scratch(s->ctx);
+  int *n2c_cnt = scratch.get<int>(ncnt), *n2f_cnt = scratch.get<int>(ncnt), *cursor = scratch.get<int>(ncnt);
+  int *ffs = scratch.get<int>(4 * (size_t)(nf > 0 ? nf : 1)), *table = scratch.get<int>(H);
+  int *ff_cnt = scratch.get<int>((size_t)(nf > 0 ? nf : 1));
+  int *flagv = scratch.get<int>(nflag), *scanv = scratch.get<int>(nflag);
 
   VAG_CUDA(cudaMemsetAsync(s->status, 0, sizeof(int), st));
   VAG_CUDA(cudaMemsetAsync(s->node_dir, 0xff, sizeof(int) * nv, st));
@@ -402,7 +398,7 @@ void symbolic_phase(System *s) {
     s->shape_start[0] = 0;
     for (int sh = 0; sh < topo::N_SHAPES; ++sh) {
       k_shape_flag<<<grid_for(nc, TB), TB, 0, st>>>(nc, s->cell_shape, sh, flagv);
-      const int cnt = scan_exclusive(flagv, scanv, nc, st);
+      const int cnt = scan_exclusive(s->ctx, flagv, scanv, nc);
       k_shape_fill<<<grid_for(nc, TB), TB, 0, st>>>(nc, s->cell_shape, sh, scanv,
                                                     s->shape_cells + s->shape_start[sh]);
       note_launches(2);
@@ -412,19 +408,21 @@ void symbolic_phase(System *s) {
     if (s->shape_start[topo::N_SHAPES] != nc) fail(VAG_EMESH, "a cell has no known shape");
   }
 
-  // fracture cells
+  // fracture cells (their count is read with the rows' below)
   k_fc_flag<<<grid_for(nc, TB), TB, 0, st>>>(nc, s->cell_ff, flagv); note_launches(1);
-  s->n_fc = scan_exclusive(flagv, scanv, nc, st);
+  scan_exclusive(s->ctx, flagv, scanv, nc, false);
   k_fc_index<<<grid_for(nc, TB), TB, 0, st>>>(nc, flagv, scanv, s->fc_index); note_launches(1);
+  int *pin = ctx_pin(s->ctx);
+  VAG_CUDA(cudaMemcpyAsync(&pin[0], scanv + nc, sizeof(int), cudaMemcpyDeviceToHost, st));
 
   // node -> cell adjacency, sorted by cell id
-  scan_exclusive(n2c_cnt, s->n2c_ptr, nv, st, false);
+  scan_exclusive(s->ctx, n2c_cnt, s->n2c_ptr, nv, false);
   VAG_CUDA(cudaMemsetAsync(cursor, 0, sizeof(int) * ncnt, st));
   k_fill_adj<<<grid_for((int64_t)nc * 8, TB), TB, 0, st>>>((int64_t)nc * 8, 8, s->cell_nodes, s->n2c_ptr,
                                                           cursor, s->n2c); note_launches(1);
   k_sort_segments<<<grid_for(nv, TB), TB, 0, st>>>(nv, s->n2c_ptr, s->n2c); note_launches(1);
   // node -> fracture-face adjacency
-  scan_exclusive(n2f_cnt, s->n2f_ptr, nv, st, false);
+  scan_exclusive(s->ctx, n2f_cnt, s->n2f_ptr, nv, false);
   if (nf) {
     VAG_CUDA(cudaMemsetAsync(cursor, 0, sizeof(int) * ncnt, st));
     k_fill_adj<<<grid_for((int64_t)nf * 4, TB), TB, 0, st>>>((int64_t)nf * 4, 4, s->ff_nodes, s->n2f_ptr,
@@ -436,33 +434,37 @@ void symbolic_phase(System *s) {
   // Krylov unknowns, contiguous per system of the batch
   k_node_flags<<<grid_for(nv, TB), TB, 0, st>>>(nv, s->node_dir, flagv);
   note_launches(1);
-  const int n_row_nodes = scan_exclusive(flagv, scanv, nv, st);
-  s->n_rows = n_row_nodes + nf;
-  s->n_row_nodes = n_row_nodes;
-  s->dof_of_row = sys_alloc<int>(s, s->n_rows);
+  scan_exclusive(s->ctx, flagv, scanv, nv, false);
   Segments &g = s->seg;
-  k_row_maps<<<grid_for(nv + nf, TB), TB, 0, st>>>(nv, nf, g.n_sys, g.d_node_start, g.d_ff_start, flagv, scanv,
-                                                   s->row_of_dof, s->dof_of_row);
-  note_launches(1);
   k_row_starts<<<grid_for(g.n_sys + 1, TB), TB, 0, st>>>(g.n_sys, g.d_node_start, g.d_ff_start, scanv,
                                                          g.d_row_start);
   note_launches(1);
   VAG_CHECK_LAUNCH();
-  g.row_start.assign(g.n_sys + 1, 0);
-  VAG_CUDA(cudaMemcpyAsync(g.row_start.data(), g.d_row_start, sizeof(int) * (g.n_sys + 1), cudaMemcpyDeviceToHost,
-                           st));
-
-  int st1 = read_status(s);
+  // one wait for the fracture cells, the rows, the row starts and the status
+  int *row_start = static_cast<int *>(ctx_stage(s->ctx, sizeof(int) * (g.n_sys + 1)));
+  VAG_CUDA(cudaMemcpyAsync(&pin[1], scanv + nv, sizeof(int), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaMemcpyAsync(&pin[2], s->status, sizeof(int), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaMemcpyAsync(row_start, g.d_row_start, sizeof(int) * (g.n_sys + 1), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaStreamSynchronize(st));
+  s->n_fc = pin[0];
+  s->n_row_nodes = pin[1];
+  s->n_rows = s->n_row_nodes + nf;
+  g.row_start.assign(row_start, row_start + g.n_sys + 1);
+  const int st1 = pin[2];
   if (st1 & ST_FFACE_NOT_FACE) fail(VAG_EMESH, "a fracture face is not a face of any cell");
   if (st1 & ST_FACE_3CELLS) fail(VAG_EMESH, "a fracture face is shared by more than two cells");
+  s->dof_of_row = sys_alloc<int>(s, s->n_rows);
+  k_row_maps<<<grid_for(nv + nf, TB), TB, 0, st>>>(nv, nf, g.n_sys, g.d_node_start, g.d_ff_start, flagv, scanv,
+                                                   s->row_of_dof, s->dof_of_row);
+  note_launches(1);
+  VAG_CHECK_LAUNCH();
 
   // CSR pattern of the eliminated system
   PatView pv{nv, nf, s->cell_nodes, s->ff_nodes, s->node_dir, s->cell_ff, s->ff_cells,
              s->n2c_ptr, s->n2c, s->n2f_ptr, s->n2f, s->row_of_dof};
   s->rowptr = sys_alloc<int>(s, (size_t)s->n_rows + 1);
   s->diag_pos = sys_alloc<int>(s, s->n_rows);
-  int *cnt;
-  VAG_CUDA(cudaMallocAsync(&cnt, sizeof(int) * ((size_t)s->n_rows + 1), st));
+  int *cnt = scratch.get<int>((size_t)s->n_rows + 1);
   k_row_count<<<grid_for(s->n_rows, 128), 128, 0, st>>>(pv, s->n_rows, s->dof_of_row, cnt, s->status); note_launches(1);
   VAG_CHECK_LAUNCH();
   if ((int64_t)s->n_rows * kMaxRowWidth > INT32_MAX) {
@@ -475,8 +477,16 @@ void symbolic_phase(System *s) {
     if (!fits_int32_indices(h.data(), h.size()))
       fail(VAG_EINVAL, "the eliminated system holds more than 2^31 - 1 stored entries (int32 indices)");
   }
-  s->nnz = scan_exclusive(cnt, s->rowptr, s->n_rows, st);
-  const int st2 = read_status(s);
+  scan_exclusive(s->ctx, cnt, s->rowptr, s->n_rows, false);
+  sell_slices(s);
+  // one wait for the entries, those of the sliced-ELL copy and the status
+  VAG_CUDA(cudaMemcpyAsync(&pin[0], s->rowptr + s->n_rows, sizeof(int), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaMemcpyAsync(&pin[1], s->slice_ptr + s->n_slices, sizeof(int), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaMemcpyAsync(&pin[2], s->status, sizeof(int), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaStreamSynchronize(st));
+  s->nnz = pin[0];
+  const int64_t sell_total = pin[1];
+  const int st2 = pin[2];
   if (st2 & ST_ROW_OVERFLOW) fail(VAG_EMESH, "an eliminated row couples too many unknowns");
   if (st2 & ST_ISOLATED) fail(VAG_EMESH, "a node belongs to no cell");
   s->col = sys_alloc<int>(s, (size_t)s->nnz);
@@ -484,16 +494,7 @@ void symbolic_phase(System *s) {
                                                       s->diag_pos); note_launches(1);
   VAG_CHECK_LAUNCH();
 
-  VAG_CUDA(cudaFreeAsync(cnt, st));
-  VAG_CUDA(cudaFreeAsync(n2c_cnt, st));
-  VAG_CUDA(cudaFreeAsync(n2f_cnt, st));
-  VAG_CUDA(cudaFreeAsync(cursor, st));
-  VAG_CUDA(cudaFreeAsync(ffs, st));
-  VAG_CUDA(cudaFreeAsync(table, st));
-  VAG_CUDA(cudaFreeAsync(ff_cnt, st));
-  VAG_CUDA(cudaFreeAsync(flagv, st));
-  VAG_CUDA(cudaFreeAsync(scanv, st));
-  VAG_CUDA(cudaStreamSynchronize(st));
+  return sell_total;
 }
 
 }  // namespace vag

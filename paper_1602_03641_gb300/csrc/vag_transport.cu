@@ -269,15 +269,15 @@ __device__ __forceinline__ bool is_dir(const TView &t, int mu) {
 // volumes all belong to one system reduces first and makes one atomic.
 __global__ void __launch_bounds__(TB) k_map_count(TView t, int n, const double *__restrict__ phi,
                                                   const int *__restrict__ cv_sys, int *__restrict__ cnt,
-                                                  unsigned long long *dt_bits) {
+                                                  unsigned long long *dt_bits, unsigned long long *total) {
   const int mu = blockIdx.x * TB + threadIdx.x;
   unsigned long long bits = ~0ull;   // no bound
   int sys = -1;
+  int c = 0;
   if (mu < n) {
     if (is_dir(t, mu)) {
       cnt[mu] = 0;
     } else {
-      int c = 0;
       double out = 0.0;
       for_edges(t, mu, [&](double Fin, int) {
         if (Fin > 0.0) ++c;
@@ -288,6 +288,9 @@ __global__ void __launch_bounds__(TB) k_map_count(TView t, int n, const double *
       if (out > 0.0) bits = (unsigned long long)__double_as_longlong(phi[mu] / out);
     }
   }
+  // the map's entries (an integer sum: any order)
+  const unsigned inflow = __reduce_add_sync(0xffffffffu, (unsigned)c);
+  if ((threadIdx.x & 31) == 0 && inflow) atomicAdd(total, (unsigned long long)inflow);
   const int s0 = __shfl_sync(0xffffffffu, sys, 0);
   if (__all_sync(0xffffffffu, sys == s0 || sys < 0) && s0 >= 0) {
 #pragma unroll
@@ -533,24 +536,6 @@ void recover_cells_and_fluxes(System *s) {
   s->have_flux = true;
 }
 
-namespace {
-// Stream-ordered scratch allocations, released on every exit path.
-struct StreamScratch {
-  cudaStream_t st;
-  std::vector<void *> p;
-  template <class T>
-  T *get(size_t count) {
-    void *q = nullptr;
-    VAG_CUDA(cudaMallocAsync(&q, sizeof(T) * std::max<size_t>(count, 1), st));
-    p.push_back(q);
-    return static_cast<T *>(q);
-  }
-  ~StreamScratch() {
-    for (void *q : p) cudaFreeAsync(q, st);
-  }
-};
-}  // namespace
-
 // phi_m [nc], phi_f [nf], cbar [nd] already on the device.
 void transport_run(System *s, const vag_transport_opts *o, double *c_dev, vag_transport_info *info,
                    const double *phi_m, const double *phi_f, const double *cbar) {
@@ -580,31 +565,37 @@ void transport_run(System *s, const vag_transport_opts *o, double *c_dev, vag_tr
   VAG_CUDA(cudaMemsetAsync(s->status, 0, sizeof(int), st));
   k_porous<<<grid_for(n, TB), TB, 0, st>>>(t, s->phi, s->status);
   note_launches(1);
-  StreamScratch scratch{st, {}};
+  Scratch scratch(s->ctx);
   int *cnt = scratch.get<int>((size_t)nt + 1);
   int *inv = scratch.get<int>((size_t)nt + 1);
   int *slice_len = scratch.get<int>((size_t)n_slices + 1);
-  unsigned long long *dt_bits = scratch.get<unsigned long long>(ns);
+  unsigned long long *dt_bits = scratch.get<unsigned long long>((size_t)ns + 1), *total = dt_bits + ns;
   VAG_CUDA(cudaMemsetAsync(dt_bits, 0x7f, sizeof(unsigned long long) * ns, st));   // > every finite ratio
-  k_map_count<<<grid_for(nt, TB), TB, 0, st>>>(t, nt, s->phi, s->seg.cv_sys, cnt, dt_bits);
-  note_launches(1);
+  VAG_CUDA(cudaMemsetAsync(total, 0, sizeof(unsigned long long), st));
+  k_map_count<<<grid_for(nt, TB), TB, 0, st>>>(t, nt, s->phi, s->seg.cv_sys, cnt, dt_bits, total);
   k_pick_dt<<<grid_for(ns, TB), TB, 0, st>>>(ns, dt_bits, s->dts, o->cfl, o->dt);
-  note_launches(1);
-  VAG_CHECK_LAUNCH();
-  const int64_t nnz_t = scan_exclusive(cnt, inv, nt, st);   // inflow entries (inv as scratch)
-  if (read_status(s) & ST_NONPOSITIVE) fail(VAG_EINVAL, "a control volume has a non-positive porous volume");
   k_sigma_sort<<<(nt + kSigma - 1) / kSigma, kSigma, 0, st>>>(nt, cnt, s->tperm, inv, slice_len);
-  note_launches(1);
+  note_launches(3);
   VAG_CHECK_LAUNCH();
-  const int64_t n_stored = scan_exclusive(slice_len, s->tsp, n_slices, st);
-  if (n_stored < nnz_t) fail(VAG_EINVAL, "the transport map exceeds 2^31 stored entries");
+  scan_exclusive(s->ctx, slice_len, s->tsp, n_slices, false);
+  // one wait for the stored entries, the map's entries and the status
+  int *pin = ctx_pin(s->ctx);
+  VAG_CUDA(cudaMemcpyAsync(&pin[0], s->tsp + n_slices, sizeof(int), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaMemcpyAsync(&pin[1], s->status, sizeof(int), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaMemcpyAsync(&pin[2], total, sizeof(unsigned long long), cudaMemcpyDeviceToHost, st));
+  VAG_CUDA(cudaStreamSynchronize(st));
+  const int64_t n_stored = pin[0];
+  unsigned long long nnz_t = 0;
+  std::copy(&pin[2], &pin[4], reinterpret_cast<int *>(&nnz_t));
+  if (pin[1] & ST_NONPOSITIVE) fail(VAG_EINVAL, "a control volume has a non-positive porous volume");
+  if (n_stored < (int64_t)nnz_t) fail(VAG_EINVAL, "the transport map exceeds 2^31 stored entries");
   if (n_stored > s->t_cap) {
     // grow the entry arrays (kept across calls)
     s->tcol = sys_alloc<int>(s, (size_t)std::max<int64_t>(n_stored, 1));
     s->tval = sys_alloc<double>(s, (size_t)std::max<int64_t>(n_stored, 1));
     s->t_cap = n_stored;
   }
-  s->nnz_t = nnz_t;
+  s->nnz_t = (int64_t)nnz_t;
   k_map_fill<<<grid_for(nt, TB), TB, 0, st>>>(t, nt, s->phi, s->seg.cv_sys, inv, s->tsp, s->dts, s->tdiag, s->tcol,
                                               s->tval);
   note_launches(1);
@@ -662,9 +653,10 @@ void transport_run(System *s, const vag_transport_opts *o, double *c_dev, vag_tr
   VAG_CUDA(cudaEventRecord(s->ev1, st));
   k_from_slots<<<grid_for(nt, TB), TB, 0, st>>>(nt, s->tperm, c0, c_dev, n);
   note_launches(1);
-  s->dts_host.resize(2 * (size_t)ns);
-  VAG_CUDA(cudaMemcpyAsync(s->dts_host.data(), s->dts, sizeof(double) * 2 * ns, cudaMemcpyDeviceToHost, st));
+  double *dts = static_cast<double *>(ctx_stage(s->ctx, sizeof(double) * 2 * ns));
+  VAG_CUDA(cudaMemcpyAsync(dts, s->dts, sizeof(double) * 2 * ns, cudaMemcpyDeviceToHost, st));
   VAG_CUDA(cudaStreamSynchronize(st));
+  s->dts_host.assign(dts, dts + 2 * (size_t)ns);
   float ms = 0.f;
   cudaEventElapsedTime(&ms, s->ev0, s->ev1);
   // a batch reports its smallest bound and step; vag_transport_get_dts gives each
