@@ -59,15 +59,52 @@ __device__ __forceinline__ int rs_sys_of_row(int i, const int *__restrict__ star
   return lo;
 }
 
+// How the setup kernels walk a level's rows: LN lanes per row, lane l taking
+// its entries l, l + LN, ...; entry k of row i is at p0 + k stride.
+//  LN = 1, the finest level in its sliced ELL: 32 rows of a warp read entry k
+//          as one segment (in CSR, a thread per row touched 32 lines a load:
+//          maxneg to p_fill took 3.0 ms at 128^3);
+//  LN = 8, coarse levels in CSR: their rows of 40 entries are read in 64-byte
+//          segments, and a level of a few thousand rows, where a thread's
+//          serial walk of its row was all the time (60-110 us a kernel
+//          whatever the level's size), takes a fifth of it.
+template <int LN>
+struct Rows {
+  int n;
+  const int *rowptr, *slice_ptr, *col;
+  const double *val;
+  __device__ __forceinline__ int len(int i) const { return rowptr[i + 1] - rowptr[i]; }
+  __device__ __forceinline__ int first(int i) const {
+    return LN == 1 ? slice_ptr[i >> 5] + (i & 31) : rowptr[i];
+  }
+  static constexpr int stride = LN == 1 ? 32 : 1;
+  // row of this thread (n or more: none) and its lane in the row
+  static __device__ __forceinline__ int row() { return (int)((blockIdx.x * (unsigned)TB + threadIdx.x) / LN); }
+  static __device__ __forceinline__ int lane() { return threadIdx.x & (LN - 1); }
+};
+// combine over the lanes of a row (every lane of the warp calls it)
+template <int LN, class T, class F>
+__device__ __forceinline__ T over_lanes(T v, F &&f) {
+#pragma unroll
+  for (int o = LN / 2; o >= 1; o /= 2) v = f(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+
 // largest negative coupling -a_ik over k != i (0 when there is none)
-__global__ void k_rs_maxneg(int n, const int *__restrict__ rowptr, const int *__restrict__ col,
-                            const double *__restrict__ val, double *__restrict__ maxneg) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+template <int LN>
+__global__ void __launch_bounds__(TB) k_rs_maxneg(Rows<LN> A, double *__restrict__ maxneg) {
+  const int i = A.row(), l = A.lane();
   double m = 0.0;
-  for (int k = rowptr[i]; k < rowptr[i + 1]; ++k)
-    if (col[k] != i && -val[k] > m) m = -val[k];
-  maxneg[i] = m;
+  if (i < A.n) {
+    const int len = A.len(i), p0 = A.first(i);
+    for (int k = l; k < len; k += LN) {
+      const int p = p0 + k * A.stride;
+      const double a = -A.val[p];
+      if (A.col[p] != i && a > m) m = a;
+    }
+  }
+  m = over_lanes<LN>(m, [](double x, double y) { return x > y ? x : y; });
+  if (i < A.n && l == 0) maxneg[i] = m;
 }
 
 // i depends strongly on j through the entry a (= a_ij = a_ji)
@@ -77,210 +114,268 @@ __device__ __forceinline__ bool rs_strong(double a, double maxneg_row) {
 
 // state: 0 undecided, 1 coarse, -1 fine, -2 fine without strong connections
 // (interpolates from nothing), -3 row of a system solved densely here
-__global__ void k_rs_init(int n, const int *__restrict__ rowptr, const int *__restrict__ col,
-                          const double *__restrict__ val, const double *__restrict__ maxneg,
-                          const uint8_t *__restrict__ skip, const int *__restrict__ sys_start, int n_sys,
-                          unsigned long long *__restrict__ key, int8_t *__restrict__ state,
-                          uint8_t *__restrict__ sflag) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  if (skip[i]) {
+template <int LN>
+__global__ void __launch_bounds__(TB) k_rs_init(Rows<LN> A, const double *__restrict__ maxneg,
+                                                const uint8_t *__restrict__ skip, const int *__restrict__ sys_start,
+                                                int n_sys, unsigned long long *__restrict__ key,
+                                                int8_t *__restrict__ state, uint8_t *__restrict__ sflag) {
+  const int i = A.row(), l = A.lane();
+  const bool valid = i < A.n;
+  const bool sk = valid && skip[i];
+  int depends = 0, infl = 0;
+  if (valid) {
+    const int len = A.len(i), p0 = A.first(i);
+    const double mi = maxneg[i];
+    for (int k = l; k < len; k += LN) {
+      const int p = p0 + k * A.stride, j = A.col[p];
+      uint8_t f = 0;
+      if (j != i && !sk) {
+        const double a = A.val[p];
+        const bool dij = rs_strong(a, mi);          // i depends on j
+        const bool dji = rs_strong(a, maxneg[j]);   // j depends on i
+        depends |= dij;
+        infl += dji;
+        f = (uint8_t)(dij | (dji << 1));
+      }
+      sflag[p] = f;   // the strength of the entry, both ways, for the PMIS rounds
+    }
+  }
+  depends = over_lanes<LN>(depends, [](int x, int y) { return x | y; });
+  infl = over_lanes<LN>(infl, [](int x, int y) { return x + y; });
+  if (!valid || l != 0) return;
+  if (sk) {
     key[i] = 0;
     state[i] = -3;
-    for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) sflag[k] = 0;
     return;
   }
-  bool depends = false;
-  unsigned infl = 0;
-  for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) {
-    const int j = col[k];
-    uint8_t f = 0;
-    if (j != i) {
-      const bool dij = rs_strong(val[k], maxneg[i]);   // i depends on j
-      const bool dji = rs_strong(val[k], maxneg[j]);   // j depends on i
-      depends |= dij;
-      infl += dji;
-      f = (uint8_t)(dij | (dji << 1));
-    }
-    sflag[k] = f;   // the strength of the entry, both ways, for the PMIS rounds
-  }
   const int loc = i - sys_start[rs_sys_of_row(i, sys_start, n_sys)];
-  key[i] = ((unsigned long long)(infl < 65535u ? infl : 65535u) << 48) |
+  key[i] = ((unsigned long long)(infl < 65535 ? infl : 65535) << 48) |
            ((unsigned long long)(rs_hash((uint32_t)loc) & 0xffffu) << 32) | (uint32_t)loc;
   state[i] = (!depends && infl == 0) ? -2 : (infl == 0 ? -1 : 0);
 }
 
 // PMIS round, first half: undecided rows that are the largest among their
 // undecided strong neighbours become coarse
-__global__ void k_rs_pmis_c(int n, const int *__restrict__ rowptr, const int *__restrict__ col,
-                            const uint8_t *__restrict__ sflag, const unsigned long long *__restrict__ key,
-                            const int8_t *__restrict__ st_in, int8_t *__restrict__ st_out, int *undecided) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) *undecided = 0;   // counted by the round's second half
-  if (i >= n) return;
-  const int8_t s = st_in[i];
-  if (s != 0) {
-    st_out[i] = s;
-    return;
+template <int LN>
+__global__ void __launch_bounds__(TB) k_rs_pmis_c(Rows<LN> A, const uint8_t *__restrict__ sflag,
+                                                  const unsigned long long *__restrict__ key,
+                                                  const int8_t *__restrict__ st_in, int8_t *__restrict__ st_out,
+                                                  int *undecided) {
+  const int i = A.row(), l = A.lane();
+  if (i == 0 && l == 0) *undecided = 0;   // counted by the round's second half
+  const int8_t s = i < A.n ? st_in[i] : (int8_t)1;
+  int top = 1;
+  if (s == 0) {
+    const unsigned long long ki = key[i];
+    const int len = A.len(i), p0 = A.first(i);
+    for (int k = l; k < len && top; k += LN) {
+      const int p = p0 + k * A.stride;
+      if (!sflag[p]) continue;   // not strong either way (or the diagonal)
+      const int j = A.col[p];
+      if (st_in[j] == 0 && key[j] > ki) top = 0;
+    }
   }
-  const unsigned long long ki = key[i];
-  bool top = true;
-  for (int k = rowptr[i]; k < rowptr[i + 1] && top; ++k) {
-    if (!sflag[k]) continue;   // not strong either way (or the diagonal)
-    const int j = col[k];
-    if (st_in[j] == 0 && key[j] > ki) top = false;
-  }
-  st_out[i] = top ? 1 : 0;
+  top = over_lanes<LN>(top, [](int x, int y) { return x & y; });
+  if (i < A.n && l == 0) st_out[i] = s != 0 ? s : (int8_t)top;
 }
 
 // second half: undecided rows that depend on a coarse row become fine; the
 // rest are counted
-__global__ void k_rs_pmis_f(int n, const int *__restrict__ rowptr, const int *__restrict__ col,
-                            const uint8_t *__restrict__ sflag, const int8_t *__restrict__ st_in,
-                            int8_t *__restrict__ st_out, int *undecided) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int8_t o = 1;
-  if (i < n) {
-    const int8_t s = st_in[i];
-    o = s;
-    if (s == 0) {
-      for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) {
-        if ((sflag[k] & 1) && st_in[col[k]] == 1) {   // i depends on a coarse row
-          o = -1;
-          break;
-        }
-      }
+template <int LN>
+__global__ void __launch_bounds__(TB) k_rs_pmis_f(Rows<LN> A, const uint8_t *__restrict__ sflag,
+                                                  const int8_t *__restrict__ st_in, int8_t *__restrict__ st_out,
+                                                  int *undecided) {
+  const int i = A.row(), l = A.lane();
+  const int8_t s = i < A.n ? st_in[i] : (int8_t)1;
+  int fine = 0;
+  if (s == 0) {
+    const int len = A.len(i), p0 = A.first(i);
+    for (int k = l; k < len && !fine; k += LN) {
+      const int p = p0 + k * A.stride;
+      fine = (sflag[p] & 1) && st_in[A.col[p]] == 1;   // i depends on a coarse row
     }
-    st_out[i] = o;
   }
+  fine = over_lanes<LN>(fine, [](int x, int y) { return x | y; });
+  if (i < A.n && l == 0) st_out[i] = s != 0 ? s : (int8_t)-fine;
   // one atomic per warp for the rows still undecided
-  const unsigned m = __ballot_sync(0xffffffffu, o == 0);
+  const unsigned m = __ballot_sync(0xffffffffu, l == 0 && s == 0 && !fine);
   if ((threadIdx.x & 31) == 0 && m) atomicAdd(undecided, __popc(m));
 }
 
 // second pass: a fine row that depends on rows but on no coarse one becomes
 // coarse
-__global__ void k_rs_second_pass(int n, const int *__restrict__ rowptr, const int *__restrict__ col,
-                                 const double *__restrict__ val, const double *__restrict__ maxneg,
-                                 const int8_t *__restrict__ st_in, int8_t *__restrict__ st_out,
-                                 int *__restrict__ cflag) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  int8_t s = st_in[i];
+template <int LN>
+__global__ void __launch_bounds__(TB) k_rs_second_pass(Rows<LN> A, const uint8_t *__restrict__ sflag,
+                                                       const int8_t *__restrict__ st_in, int8_t *__restrict__ st_out,
+                                                       int *__restrict__ cflag) {
+  const int i = A.row(), l = A.lane();
+  int8_t s = i < A.n ? st_in[i] : (int8_t)1;
+  int has = 0;   // 1: depends on some row, 2: on a coarse one
   if (s == -1) {
-    bool depends = false, has_c = false;
-    for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) {
-      const int j = col[k];
-      if (j == i || !rs_strong(val[k], maxneg[i])) continue;
-      depends = true;
-      has_c |= st_in[j] == 1;
+    const int len = A.len(i), p0 = A.first(i);
+    for (int k = l; k < len; k += LN) {
+      const int p = p0 + k * A.stride;
+      if (sflag[p] & 1) has |= st_in[A.col[p]] == 1 ? 3 : 1;
     }
-    if (depends && !has_c) s = 1;
   }
+  has = over_lanes<LN>(has, [](int x, int y) { return x | y; });
+  if (i >= A.n || l != 0) return;
+  if (has == 1) s = 1;
   st_out[i] = s;
   cflag[i] = s == 1;
 }
 
-// the chosen coarse neighbours of fine row i: its strong coarse neighbours,
-// at most kPmax of them with the largest |a_ij| (ties by smaller index);
-// returned as CSR positions in CSR order
-__device__ __forceinline__ int rs_choose(int i, const int *__restrict__ rowptr, const int *__restrict__ col,
-                                         const double *__restrict__ val, const double *__restrict__ maxneg,
-                                         const int8_t *__restrict__ st, int (&pick)[kPmax]) {
-  int m = 0;
-  for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) {
-    const int j = col[k];
-    if (j == i || st[j] != 1 || !rs_strong(val[k], maxneg[i])) continue;
-    const double a = fabs(val[k]);
-    if (m < kPmax) {
-      pick[m++] = k;
-      continue;
-    }
-    // replace the weakest pick (on a tie the one of larger index) if this
-    // one is strictly stronger
-    int wq = 0;
-    for (int q = 1; q < kPmax; ++q) {
-      const double aq = fabs(val[pick[q]]), aw = fabs(val[pick[wq]]);
-      if (aq < aw || (aq == aw && col[pick[q]] > col[pick[wq]])) wq = q;
-    }
-    if (a > fabs(val[pick[wq]])) pick[wq] = k;
-  }
-  for (int p = 1; p < m; ++p)   // CSR order
-    for (int q = p; q > 0 && pick[q - 1] > pick[q]; --q) {
-      const int t = pick[q];
-      pick[q] = pick[q - 1];
-      pick[q - 1] = t;
-    }
-  return m;
-}
-
-__global__ void k_rs_p_count(int n, const int *__restrict__ rowptr, const int *__restrict__ col,
-                             const double *__restrict__ val, const double *__restrict__ maxneg,
-                             const int8_t *__restrict__ st, int *__restrict__ cnt) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int8_t s = st[i];
-  int c = 0;
-  if (s == 1) {
-    c = 1;
-  } else if (s == -1) {
-    int pick[kPmax];
-    c = rs_choose(i, rowptr, col, val, maxneg, st, pick);
-  }
-  cnt[i] = c;
-}
-
-__global__ void k_rs_p_fill(int n, const int *__restrict__ rowptr, const int *__restrict__ col,
-                            const double *__restrict__ val, const double *__restrict__ maxneg,
-                            const int8_t *__restrict__ st, const int *__restrict__ cidx,
-                            const int *__restrict__ prow, int *__restrict__ pcol, double *__restrict__ pval,
-                            int *status) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int8_t s = st[i];
-  const int o = prow[i];
-  if (s == 1) {
-    pcol[o] = cidx[i];
-    pval[o] = 1.0;
-    return;
-  }
-  if (s != -1) return;
-  int pick[kPmax];
-  const int m = rs_choose(i, rowptr, col, val, maxneg, st, pick);
-  if (m != prow[i + 1] - o) {
-    atomicOr(status, ST_BAD_INDEX);
-    return;
-  }
+// P's row i before the coarse numbering is known: the entries it takes (a
+// coarse row: itself; a fine row: its strong coarse neighbours, at most kPmax
+// of them with the largest |a_ij|, ties by position) as positions in the
+// level's entry array, in row order, and (alpha_i, a_ii + sum of the positive
+// couplings), the sums taken in row order whatever LN.
+template <int LN>
+__global__ void __launch_bounds__(TB) k_rs_choose(Rows<LN> A, const uint8_t *__restrict__ sflag,
+                                                  const int8_t *__restrict__ st, int *__restrict__ cnt,
+                                                  int4 *__restrict__ picks, double2 *__restrict__ factor,
+                                                  int *status) {
+  static_assert(kPmax == 4, "picks of a row are one int4");
+  const int i = A.row(), l = A.lane();
+  const int8_t s = i < A.n ? st[i] : (int8_t)0;
   double aii = 0.0, neg = 0.0, pos = 0.0;
-  for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) {
-    const double a = val[k];
-    if (col[k] == i) aii += a;
-    else if (a < 0.0) neg += a;
-    else pos += a;
+  int pk[kPmax];
+  double pa[kPmax];
+  int m = 0;
+  const int len = s == -1 ? A.len(i) : 0, p0 = s == -1 ? A.first(i) : 0;
+  const int rounds = LN == 1 ? len : __reduce_max_sync(0xffffffffu, (len + LN - 1) / LN);
+  for (int k = l, round = 0; round < rounds; ++round, k += LN) {
+    double a = 0.0;
+    int kind = 3;   // 0 diagonal, 1 negative, 2 positive coupling, 3 none
+    if (k < len) {
+      const int p = p0 + k * A.stride, j = A.col[p];
+      a = A.val[p];
+      kind = j == i ? 0 : a < 0.0 ? 1 : 2;
+      if ((sflag[p] & 1) && st[j] == 1 && !(m == kPmax && !(a < pa[kPmax - 1]))) {
+        // into this lane's kPmax strongest (a < 0: the smallest values), strongest first
+        int q = m < kPmax ? m++ : kPmax - 1;
+#pragma unroll
+        for (int t = kPmax - 1; t > 0; --t)
+          if (t == q) {
+            if (!(a < pa[t - 1])) {
+              pk[t] = k;
+              pa[t] = a;
+              q = -1;
+            } else {
+              pk[t] = pk[t - 1];
+              pa[t] = pa[t - 1];
+              q = t - 1;
+            }
+          }
+        if (q == 0) {
+          pk[0] = k;
+          pa[0] = a;
+        }
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < LN; ++t) {   // the lanes' entries in row order
+      const double at = LN == 1 ? a : __shfl_sync(0xffffffffu, a, t, LN);
+      const int kt = LN == 1 ? kind : __shfl_sync(0xffffffffu, kind, t, LN);
+      if (kt == 0) aii += at;
+      else if (kt == 1) neg += at;
+      else if (kt == 2) pos += at;
+    }
   }
   double cneg = 0.0;
-  for (int q = 0; q < m; ++q) cneg += val[pick[q]];
+  if (LN > 1) {
+    // the row's kPmax strongest from the lanes' lists: kPmax rounds of the
+    // strongest head (ties by position)
+    int gk[kPmax], gm = 0;
+    double ga[kPmax];
+#pragma unroll
+    for (int t = 0; t < kPmax; ++t) {
+      double ba = m > 0 ? pa[0] : 0.0;
+      int bk = m > 0 ? pk[0] : INT_MAX;
+#pragma unroll
+      for (int o = LN / 2; o >= 1; o /= 2) {
+        const double oa = __shfl_xor_sync(0xffffffffu, ba, o);
+        const int ok = __shfl_xor_sync(0xffffffffu, bk, o);
+        if (oa < ba || (oa == ba && ok < bk)) { ba = oa; bk = ok; }
+      }
+      gk[t] = bk;
+      ga[t] = ba;
+      if (bk != INT_MAX) {
+        gm = t + 1;
+        if (m > 0 && pk[0] == bk) {   // taken from this lane's list
+#pragma unroll
+          for (int u = 0; u + 1 < kPmax; ++u) { pk[u] = pk[u + 1]; pa[u] = pa[u + 1]; }
+          --m;
+        }
+      }
+    }
+    m = gm;
+#pragma unroll
+    for (int t = 0; t < kPmax; ++t) { pk[t] = gk[t]; pa[t] = ga[t]; }
+  }
+  if (i >= A.n || l != 0) return;
+  if (s != -1) {
+    cnt[i] = s == 1;
+    return;
+  }
+  // row order
+#pragma unroll
+  for (int p = 1; p < kPmax; ++p)
+#pragma unroll
+    for (int q = p; q > 0; --q)
+      if (p < m && pk[q - 1] > pk[q]) {
+        const int t = pk[q]; pk[q] = pk[q - 1]; pk[q - 1] = t;
+        const double x = pa[q]; pa[q] = pa[q - 1]; pa[q - 1] = x;
+      }
+#pragma unroll
+  for (int q = 0; q < kPmax; ++q)
+    if (q < m) cneg += pa[q];
   const double diag = aii + pos;
   if (!(diag > 0.0) || !(cneg < 0.0)) {
     atomicOr(status, ST_NONPOSITIVE);
-    return;
+    m = 0;
   }
-  const double alpha = neg / cneg;
-  for (int q = 0; q < m; ++q) {
-    pcol[o + q] = cidx[col[pick[q]]];
-    pval[o + q] = -alpha * val[pick[q]] / diag;
-  }
+  int4 o;
+  o.x = m > 0 ? p0 + pk[0] * A.stride : 0;
+  o.y = m > 1 ? p0 + pk[1] * A.stride : 0;
+  o.z = m > 2 ? p0 + pk[2] * A.stride : 0;
+  o.w = m > 3 ? p0 + pk[3] * A.stride : 0;
+  picks[i] = o;
+  factor[i] = make_double2(neg / cneg, diag);
+  cnt[i] = m;
 }
 
-// R = P^T: counts per coarse row, entries placed by an atomic cursor, then
-// each row sorted by fine index (so its content does not depend on the order
-// of the atomics)
-__global__ void k_rs_r_count(int n, const int *__restrict__ prow, const int *__restrict__ pcol, int *rcnt) {
+// P's rows, and R's row counts
+__global__ void k_rs_p_fill(int n, const int *__restrict__ acol, const double *__restrict__ aval,
+                            const int8_t *__restrict__ st, const int *__restrict__ cidx, const int4 *__restrict__ picks,
+                            const double2 *__restrict__ factor, const int *__restrict__ prow, int *__restrict__ pcol,
+                            double *__restrict__ pval, int *rcnt) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  for (int k = prow[i]; k < prow[i + 1]; ++k) atomicAdd(&rcnt[pcol[k]], 1);
+  const int o = prow[i], m = prow[i + 1] - o;
+  if (m == 0) return;
+  if (st[i] == 1) {
+    const int I = cidx[i];
+    pcol[o] = I;
+    pval[o] = 1.0;
+    atomicAdd(&rcnt[I], 1);
+    return;
+  }
+  const int4 pk = picks[i];
+  const double alpha = factor[i].x, diag = factor[i].y;
+  const int p[kPmax] = {pk.x, pk.y, pk.z, pk.w};
+#pragma unroll
+  for (int q = 0; q < kPmax; ++q)
+    if (q < m) {
+      const int I = cidx[acol[p[q]]];
+      pcol[o + q] = I;
+      pval[o + q] = -alpha * aval[p[q]] / diag;
+      atomicAdd(&rcnt[I], 1);
+    }
 }
 
+// R = P^T: entries placed by an atomic cursor, then each row sorted by fine
+// index (so its content does not depend on the order of the atomics)
 __global__ void k_rs_r_fill(int n, const int *__restrict__ prow, const int *__restrict__ pcol,
                             const double *__restrict__ pval, const int *__restrict__ rrow, int *cursor,
                             int *__restrict__ rcol, double *__restrict__ rval) {
@@ -294,14 +389,30 @@ __global__ void k_rs_r_fill(int n, const int *__restrict__ prow, const int *__re
   }
 }
 
-__global__ void k_rs_r_sort(int nc, const int *__restrict__ rrow, int *rcol, double *rval) {
-  const int I = blockIdx.x * blockDim.x + threadIdx.x;
-  if (I >= nc) return;
-  for (int p = rrow[I] + 1; p < rrow[I + 1]; ++p) {
+// One warp per row of R, entries in registers, their places by counting the
+// smaller indices of the row (rows of up to 32 entries; longer ones, which
+// direct interpolation hardly makes, by insertion in one lane).
+__global__ void __launch_bounds__(TB) k_rs_r_sort(int nc, const int *__restrict__ rrow, int *rcol, double *rval) {
+  const int I = blockIdx.x * (TB / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (I >= nc) return;   // whole warps
+  const int b = rrow[I], m = rrow[I + 1] - b;
+  if (m <= 32) {
+    const int c = lane < m ? rcol[b + lane] : INT_MAX;
+    const double v = lane < m ? rval[b + lane] : 0.0;
+    int rank = 0;
+    for (int q = 0; q < m; ++q) rank += __shfl_sync(0xffffffffu, c, q) < c;
+    if (lane < m) {   // every lane has read its entry (the shuffles above)
+      rcol[b + rank] = c;
+      rval[b + rank] = v;
+    }
+    return;
+  }
+  if (lane != 0) return;
+  for (int p = b + 1; p < b + m; ++p) {
     const int c = rcol[p];
     const double v = rval[p];
     int q = p - 1;
-    while (q >= rrow[I] && rcol[q] > c) {
+    while (q >= b && rcol[q] > c) {
       rcol[q + 1] = rcol[q];
       rval[q + 1] = rval[q];
       --q;
@@ -454,15 +565,18 @@ static int rap_blocks(int nrows, int warps) {
   return std::max(1, std::min(want, cap));
 }
 
+// Pack the rows, one warp per row (a row a thread: 1.0 ms of the 128^3 setup).
 template <int CAP>
-__global__ void k_rs_compact(int nc, const int *__restrict__ tcol, const double *__restrict__ tval,
-                             const int *__restrict__ rowptr, int *__restrict__ col, double *__restrict__ val) {
-  const int I = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(TB) k_rs_compact(int nc, const int *__restrict__ tcol,
+                                                   const double *__restrict__ tval, const int *__restrict__ rowptr,
+                                                   int *__restrict__ col, double *__restrict__ val) {
+  const int I = blockIdx.x * (TB / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (I >= nc) return;
   const size_t base = (size_t)I * CAP;
-  for (int q = 0; q < rowptr[I + 1] - rowptr[I]; ++q) {
-    col[rowptr[I] + q] = tcol[base + q];
-    val[rowptr[I] + q] = tval[base + q];
+  const int o = rowptr[I], m = rowptr[I + 1] - o;
+  for (int q = lane; q < m; q += 32) {
+    col[o + q] = tcol[base + q];
+    val[o + q] = tval[base + q];
   }
 }
 
@@ -499,10 +613,24 @@ void rs_coarsen(System *s, AmgLevel &L, AmgLevel &C, const std::function<void *(
   int8_t *sb = static_cast<int8_t *>(tmp(std::max(n, 1)));
   int *undecided = static_cast<int *>(tmp(sizeof(int)));
   const int g = grid_for(n, TB);
-  k_rs_maxneg<<<g, TB, 0, st>>>(n, L.rowptr, L.col, L.val, maxneg);
-  uint8_t *sflag = static_cast<uint8_t *>(tmp((size_t)std::max<int64_t>(L.nnz, 1)));
-  k_rs_init<<<g, TB, 0, st>>>(n, L.rowptr, L.col, L.val, maxneg, L.skip, L.d_sys_start, ns, key, sa, sflag);
-  note_launches(2);
+  // the finest level (the system's own matrix) is walked in its sliced ELL
+  const bool sell = L.slice_ptr != nullptr;
+  const int64_t entries = sell ? L.sell_nnz : L.nnz;
+  const int *acol = sell ? L.scol : L.col;
+  const double *aval = sell ? L.sval : L.val;
+  const Rows<1> A1{n, L.rowptr, L.slice_ptr, acol, aval};
+  const Rows<8> A8{n, L.rowptr, nullptr, acol, aval};
+  const int ga = sell ? g : grid_for(8 * (int64_t)n, TB);
+#define RS_LAUNCH(kernel, ...)                                                       \
+  do {                                                                               \
+    if (sell) kernel<1><<<ga, TB, 0, st>>>(A1, __VA_ARGS__);                         \
+    else kernel<8><<<ga, TB, 0, st>>>(A8, __VA_ARGS__);                              \
+    note_launches(1);                                                                \
+  } while (0)
+  uint8_t *sflag = static_cast<uint8_t *>(tmp((size_t)std::max<int64_t>(entries, 1)));
+  VAG_CUDA(cudaMemsetAsync(s->status, 0, sizeof(int), st));   // checked after the Galerkin product
+  RS_LAUNCH(k_rs_maxneg, maxneg);
+  RS_LAUNCH(k_rs_init, maxneg, L.skip, L.d_sys_start, ns, key, sa, sflag);
   VAG_CHECK_LAUNCH();
   trace_mark(st, "  classical: strength + measure");
   // PMIS rounds (two kernels each, states ping-pong).  The second pass, P's
@@ -514,49 +642,47 @@ void rs_coarsen(System *s, AmgLevel &L, AmgLevel &C, const std::function<void *(
   int *cflag = static_cast<int *>(tmp(4 * (size_t)std::max(n, 1)));
   int *cidx = static_cast<int *>(tmp(4 * ((size_t)n + 1)));
   int *pcnt = static_cast<int *>(tmp(4 * ((size_t)n + 1)));
+  int4 *picks = static_cast<int4 *>(tmp(16 * (size_t)std::max(n, 1)));
+  double2 *factor = static_cast<double2 *>(tmp(16 * (size_t)std::max(n, 1)));
   L.prow = static_cast<int *>(alloc(4 * ((size_t)n + 1)));
   const int8_t *state = sb;
   bool finished = false;
   for (int r = 0, next = n > 2000 ? 8 : 4; r < kMaxRounds && !finished; next += 4) {
     for (; r < next; ++r) {
-      k_rs_pmis_c<<<g, TB, 0, st>>>(n, L.rowptr, L.col, sflag, key, sa, sb, undecided);
-      k_rs_pmis_f<<<g, TB, 0, st>>>(n, L.rowptr, L.col, sflag, sb, sa, undecided);
-      note_launches(2);
+      RS_LAUNCH(k_rs_pmis_c, sflag, key, sa, sb, undecided);
+      RS_LAUNCH(k_rs_pmis_f, sflag, sb, sa, undecided);
     }
     trace_mark(st, "  classical: PMIS rounds");
-    k_rs_second_pass<<<g, TB, 0, st>>>(n, L.rowptr, L.col, L.val, maxneg, sa, sb, cflag);
+    RS_LAUNCH(k_rs_second_pass, sflag, sa, sb, cflag);
     scan_exclusive(s->ctx, cflag, cidx, n, false);
-    k_rs_p_count<<<g, TB, 0, st>>>(n, L.rowptr, L.col, L.val, maxneg, state, pcnt);
+    RS_LAUNCH(k_rs_choose, sflag, state, pcnt, picks, factor, s->status);
     scan_exclusive(s->ctx, pcnt, L.prow, n, false);
-    note_launches(2);
     VAG_CUDA(cudaMemcpyAsync(&pin[0], cidx + n, sizeof(int), cudaMemcpyDeviceToHost, st));
     VAG_CUDA(cudaMemcpyAsync(&pin[1], L.prow + n, sizeof(int), cudaMemcpyDeviceToHost, st));
     VAG_CUDA(cudaMemcpyAsync(&pin[2], undecided, sizeof(int), cudaMemcpyDeviceToHost, st));
     VAG_CUDA(cudaStreamSynchronize(st));
     finished = pin[2] == 0;
+    if (!finished) VAG_CUDA(cudaMemsetAsync(s->status, 0, sizeof(int), st));
   }
+#undef RS_LAUNCH
   if (!finished) fail(VAG_ECUDA, "AMG: the PMIS splitting did not finish");
   const int nc = pin[0];
   L.p_nnz = pin[1];
   L.pcol = static_cast<int *>(alloc(4 * (size_t)std::max<int64_t>(L.p_nnz, 1)));
   L.pval = static_cast<double *>(alloc(8 * (size_t)std::max<int64_t>(L.p_nnz, 1)));
-  VAG_CUDA(cudaMemsetAsync(s->status, 0, sizeof(int), st));   // checked after the Galerkin product
-  k_rs_p_fill<<<g, TB, 0, st>>>(n, L.rowptr, L.col, L.val, maxneg, state, cidx, L.prow, L.pcol, L.pval, s->status);
-  note_launches(1);
-  // R = P^T
-  int *rcnt = static_cast<int *>(tmp(4 * ((size_t)nc + 1)));
-  int *cursor = static_cast<int *>(tmp(4 * ((size_t)nc + 1)));
+  // R = P^T (its row counts come with P)
+  int *rcnt = static_cast<int *>(tmp(8 * ((size_t)nc + 1)));
+  int *cursor = rcnt + nc + 1;
   L.rrow = static_cast<int *>(alloc(4 * ((size_t)nc + 1)));
-  VAG_CUDA(cudaMemsetAsync(rcnt, 0, 4 * ((size_t)nc + 1), st));
-  VAG_CUDA(cudaMemsetAsync(cursor, 0, 4 * ((size_t)nc + 1), st));
-  k_rs_r_count<<<g, TB, 0, st>>>(n, L.prow, L.pcol, rcnt);
+  VAG_CUDA(cudaMemsetAsync(rcnt, 0, 8 * ((size_t)nc + 1), st));
+  k_rs_p_fill<<<g, TB, 0, st>>>(n, acol, aval, state, cidx, picks, factor, L.prow, L.pcol, L.pval, rcnt);
   note_launches(1);
   scan_exclusive(s->ctx, rcnt, L.rrow, nc, false);
   L.r_nnz = L.p_nnz;
   L.rcol = static_cast<int *>(alloc(4 * (size_t)std::max<int64_t>(L.r_nnz, 1)));
   L.rval = static_cast<double *>(alloc(8 * (size_t)std::max<int64_t>(L.r_nnz, 1)));
   k_rs_r_fill<<<g, TB, 0, st>>>(n, L.prow, L.pcol, L.pval, L.rrow, cursor, L.rcol, L.rval);
-  k_rs_r_sort<<<grid_for(nc, TB), TB, 0, st>>>(nc, L.rrow, L.rcol, L.rval);
+  k_rs_r_sort<<<grid_for(nc, TB / 32), TB, 0, st>>>(nc, L.rrow, L.rcol, L.rval);
   note_launches(2);
   VAG_CHECK_LAUNCH();
   L.nc = nc;
@@ -590,14 +716,13 @@ void rs_coarsen(System *s, AmgLevel &L, AmgLevel &C, const std::function<void *(
   C.nnz = pin[0];
   {
     const int stv = pin[1];
-    if (stv & ST_BAD_INDEX) fail(VAG_ECUDA, "AMG: internal interpolation count mismatch");
     if (stv & ST_ROW_OVERFLOW) fail(VAG_EMESH, "AMG: a coarse row couples too many coarse rows");
     if (stv & ST_NONPOSITIVE)
       fail(VAG_EINVAL, "AMG: a fine row has no usable coarse couplings or a coarse diagonal is not positive");
   }
   C.col = static_cast<int *>(alloc(4 * (size_t)std::max<int64_t>(C.nnz, 1)));
   C.val = static_cast<double *>(alloc(8 * (size_t)std::max<int64_t>(C.nnz, 1)));
-  k_rs_compact<kRapCap><<<grid_for(nc, TB), TB, 0, st>>>(nc, tcol, tval, C.rowptr, C.col, C.val);
+  k_rs_compact<kRapCap><<<grid_for(nc, TB / 32), TB, 0, st>>>(nc, tcol, tval, C.rowptr, C.col, C.val);
   note_launches(1);
   trace_mark(st, "  classical: Galerkin R A P");
   VAG_CHECK_LAUNCH();
