@@ -574,26 +574,24 @@ __global__ void __launch_bounds__(256) k_jac_csr(int n, const int *__restrict__ 
 
 // same sweep in the sliced-ELL layout (level 0), one thread per row
 template <class T, int U>
-__global__ void k_jac_sell(int n, const int *__restrict__ rowptr, const int *__restrict__ slice_ptr,
-                           const int *__restrict__ scol, const T *__restrict__ sval, const T *__restrict__ sinv,
+__global__ void k_jac_sell(int n, SellIdx ix, const T *__restrict__ sval, const T *__restrict__ sinv,
                            const T *__restrict__ b, const T *__restrict__ xin, T *__restrict__ xout,
                            const uint8_t *__restrict__ skip) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   pdl_wait();
   pdl_trigger();
   if (i >= n || skip[i]) return;
-  xout[i] = jac_row(xin[i], sinv[i], b[i], sell_row<T, U>(i, rowptr, slice_ptr, scol, sval, xin));
+  xout[i] = jac_row(xin[i], sinv[i], b[i], sell_row<T, U>(i, ix, sval, xin));
 }
 
 template <class T, int U>
-__global__ void k_resid_sell(int n, const int *__restrict__ rowptr, const int *__restrict__ slice_ptr,
-                             const int *__restrict__ scol, const T *__restrict__ sval, const T *__restrict__ b,
+__global__ void k_resid_sell(int n, SellIdx ix, const T *__restrict__ sval, const T *__restrict__ b,
                              const T *__restrict__ x, T *__restrict__ r) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   pdl_wait();
   pdl_trigger();
   if (i >= n) return;
-  r[i] = b[i] - sell_row<T, U>(i, rowptr, slice_ptr, scol, sval, x);
+  r[i] = b[i] - sell_row<T, U>(i, ix, sval, x);
 }
 
 // The last finest-level sweep of the V-cycle inside CG (FP64 CG, or the FP32
@@ -603,8 +601,7 @@ __global__ void k_resid_sell(int n, const int *__restrict__ rowptr, const int *_
 // tile of a system adding the tile partials in order and setting
 // beta = (r.z)' / (r.z) and rho = (r.z)'.
 template <class T, int U>
-__global__ void __launch_bounds__(256) k_jac_sell_rz(const int *__restrict__ rowptr, const int *__restrict__ slice_ptr,
-                                                     const int *__restrict__ scol, const T *__restrict__ sval,
+__global__ void __launch_bounds__(256) k_jac_sell_rz(SellIdx ix, const T *__restrict__ sval,
                                                      const T *__restrict__ sinv, const T *__restrict__ r,
                                                      const T *__restrict__ xin, T *__restrict__ z,
                                                      const uint8_t *__restrict__ skip, Tiles tl, double *partials,
@@ -622,7 +619,7 @@ __global__ void __launch_bounds__(256) k_jac_sell_rz(const int *__restrict__ row
     if (skip[i]) {
       zi = z[i];   // solved densely on this level
     } else {
-      zi = jac_row(xin[i], sinv[i], r[i], sell_row<T, U>(i, rowptr, slice_ptr, scol, sval, xin));
+      zi = jac_row(xin[i], sinv[i], r[i], sell_row<T, U>(i, ix, sval, xin));
       z[i] = zi;
     }
     rz = (double)fma(r[i], zi, (T)0);
@@ -1103,28 +1100,26 @@ __global__ void k_to_f64_scaled(int n, const float *__restrict__ x, const double
 }
 
 template <int U>
-__global__ void k_jac_sell_h(int n, const int *__restrict__ rowptr, const int *__restrict__ slice_ptr,
-                             const int *__restrict__ scol, const __half *__restrict__ sval,
+__global__ void k_jac_sell_h(int n, SellIdx ix, const __half *__restrict__ sval,
                              const float *__restrict__ sinv, const float *__restrict__ b,
                              const float *__restrict__ xin, float *__restrict__ xout, const uint8_t *__restrict__ skip) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   pdl_wait();
   pdl_trigger();
   if (i >= n || skip[i]) return;
-  xout[i] = jac_row(xin[i], sinv[i], b[i], sell_row<float, U, __half>(i, rowptr, slice_ptr, scol, sval, xin));
+  xout[i] = jac_row(xin[i], sinv[i], b[i], sell_row<float, U, __half>(i, ix, sval, xin));
 }
 
 // unscaled residual b - A x = S^-1 (b~ - h x~) for the restriction
 template <int U>
-__global__ void k_resid_sell_h(int n, const int *__restrict__ rowptr, const int *__restrict__ slice_ptr,
-                               const int *__restrict__ scol, const __half *__restrict__ sval,
+__global__ void k_resid_sell_h(int n, SellIdx ix, const __half *__restrict__ sval,
                                const float *__restrict__ s0f, const float *__restrict__ b,
                                const float *__restrict__ x, float *__restrict__ r) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   pdl_wait();
   pdl_trigger();
   if (i >= n) return;
-  r[i] = s0f[i] * (b[i] - sell_row<float, U, __half>(i, rowptr, slice_ptr, scol, sval, x));
+  r[i] = s0f[i] * (b[i] - sell_row<float, U, __half>(i, ix, sval, x));
 }
 
 // a system solved densely on the finest level, in scaled variables:
@@ -1584,17 +1579,17 @@ static bool vcycle(System *s, int lvl, const T *b, T *x, cudaStream_t st, bool c
   constexpr int LN = row_lanes<T>();
   const int gL = grid_for(n, 256 / LN);   // LN lanes per row
   // finest level: the autotuned loads in flight of the sliced-ELL row loop
-  auto jac_sell = s->sell_u == 2 ? k_jac_sell<T, 2> : s->sell_u == 8 ? k_jac_sell<T, 8> : k_jac_sell<T, 4>;
-  auto resid_sell = s->sell_u == 2 ? k_resid_sell<T, 2> : s->sell_u == 8 ? k_resid_sell<T, 8> : k_resid_sell<T, 4>;
+  auto jac_sell = sell_pick(s, s->sell_u, [](auto u) { return k_jac_sell<T, decltype(u)::value>; });
+  auto resid_sell = sell_pick(s, s->sell_u, [](auto u) { return k_resid_sell<T, decltype(u)::value>; });
   const bool h16 = sizeof(T) == 4 && lvl == 0 && A.f16;   // scaled FP16 finest level
-  auto jac_h = s->sell_u == 2 ? k_jac_sell_h<2> : s->sell_u == 8 ? k_jac_sell_h<8> : k_jac_sell_h<4>;
+  auto jac_h = sell_pick(s, s->sell_u, [](auto u) { return k_jac_sell_h<decltype(u)::value>; });
   if (h16) {
     const float *bb = (const float *)b;
     float *xx = (float *)x, *tt = A.levels[0].t32;
     const LV<float> c32 = lv<float>(s, C);
-    auto resid_h = s->sell_u == 2 ? k_resid_sell_h<2> : s->sell_u == 8 ? k_resid_sell_h<8> : k_resid_sell_h<4>;
+    auto resid_h = sell_pick(s, s->sell_u, [](auto u) { return k_resid_sell_h<decltype(u)::value>; });
     launch_pdl(k_jac_first<float>, g, TB, 0, st, n, bb, (const float *)A.sinv16, tt);
-    launch_pdl(resid_h, g, TB, 0, st, n, (const int *)L.rowptr, (const int *)L.slice_ptr, (const int *)L.scol,
+    launch_pdl(resid_h, g, TB, 0, st, n, sell_idx(s),
                (const __half *)A.sval16, (const float *)A.s0f, bb, (const float *)tt, L.r32);
     launch_pdl(k_restrict_first<float>, grid_for(C.n, TB), TB, 0, st, C.n, (const int *)L.mptr, (const int *)L.mem,
                (const float *)L.r32, c32.sinv, c32.b, c32.t);
@@ -1603,8 +1598,7 @@ static bool vcycle(System *s, int lvl, const T *b, T *x, cudaStream_t st, bool c
     // level 0: sliced ELL, one thread per row; one sweep from zero, t =
     // omega D_l1^-1 b, then the residual b - A t for the restriction
     if (!cg) launch_pdl(k_jac_first<T>, g, TB, 0, st, n, b, v.sinv, v.t);
-    launch_pdl(resid_sell, g, TB, 0, st, n, (const int *)L.rowptr, (const int *)L.slice_ptr,
-               (const int *)L.scol, v.sval, b, (const T *)v.t, v.r);
+    launch_pdl(resid_sell, g, TB, 0, st, n, sell_idx(s), v.sval, b, (const T *)v.t, v.r);
     if (A.classical)
       launch_pdl(k_rs_restrict<T>, grid_for(C.n, 256 / LN), 256, 0, st, C.n, (const int *)L.rrow,
                  (const int *)L.rcol, v.rv, (const T *)v.r, c.sinv, c.b, c.t);
@@ -1646,7 +1640,7 @@ static bool vcycle(System *s, int lvl, const T *b, T *x, cudaStream_t st, bool c
     float *xx = (float *)x, *tt = A.levels[0].t32;
     launch_pdl(k_prolong_scaled, g, TB, 0, st, n, (const int *)L.agg, (const float *)A.s0f,
                (const float *)A.levels[1].x32, tt);
-    launch_pdl(jac_h, g, TB, 0, st, n, (const int *)L.rowptr, (const int *)L.slice_ptr, (const int *)L.scol,
+    launch_pdl(jac_h, g, TB, 0, st, n, sell_idx(s),
                (const __half *)A.sval16, (const float *)A.sinv16, bb, (const float *)tt, xx, (const uint8_t *)L.skip);
     note_launches(2);
   } else if (lvl == 0) {
@@ -1656,17 +1650,16 @@ static bool vcycle(System *s, int lvl, const T *b, T *x, cudaStream_t st, bool c
     else
       launch_pdl(k_prolong<T>, g, TB, 0, st, n, (const int *)L.agg, (const T *)c.x, v.t);
     if (cg) {   // the last sweep forms r.z for the Krylov loop (cg_ks, cg_done)
-      auto jr = s->sell_u == 2 ? k_jac_sell_rz<T, 2> : s->sell_u == 8 ? k_jac_sell_rz<T, 8> : k_jac_sell_rz<T, 4>;
+      auto jr = sell_pick(s, s->sell_u, [](auto u) { return k_jac_sell_rz<T, decltype(u)::value>; });
       const Tiles tl{s->seg.tile_sys, s->seg.tile_row0, s->seg.tile_row1, s->seg.sys_tile0, s->seg.sys_grp0,
                      s->seg.n_tiles, s->seg.n_sys};
-      launch_pdl(jr, s->seg.n_tiles, 256, 0, st, (const int *)L.rowptr, (const int *)L.slice_ptr,
-                 (const int *)L.scol, (const T *)v.sval, (const T *)v.sinv, (const T *)b, (const T *)v.t, (T *)x,
-                 (const uint8_t *)L.skip, tl, s->partials, s->counter, cg_ks, cg_done);
+      launch_pdl(jr, s->seg.n_tiles, 256, 0, st, sell_idx(s), (const T *)v.sval, (const T *)v.sinv, (const T *)b,
+                 (const T *)v.t, (T *)x, (const uint8_t *)L.skip, tl, s->partials, s->counter, cg_ks, cg_done);
       note_launches(2);
       return true;
     }
-    launch_pdl(jac_sell, g, TB, 0, st, n, (const int *)L.rowptr, (const int *)L.slice_ptr, (const int *)L.scol,
-               v.sval, v.sinv, b, (const T *)v.t, x, (const uint8_t *)L.skip);
+    launch_pdl(jac_sell, g, TB, 0, st, n, sell_idx(s), v.sval, v.sinv, b, (const T *)v.t, x,
+               (const uint8_t *)L.skip);
     note_launches(2);
   } else if (A.classical) {
     // coarse correction x += P x_c, then two sweeps
@@ -1758,9 +1751,9 @@ double time_smoother(System *s, int reps) {
   cudaStream_t st = s->ctx->stream;
   const int n = L.n, g = grid_for(n, TB);
   if (A.f32) {
-    auto jac = s->sell_u == 2 ? k_jac_sell<float, 2> : s->sell_u == 8 ? k_jac_sell<float, 8> : k_jac_sell<float, 4>;
+    auto jac = sell_pick(s, s->sell_u, [](auto u) { return k_jac_sell<float, decltype(u)::value>; });
     auto sweep32 = [&](const float *xin, float *xout) {
-      launch_pdl(jac, g, TB, 0, st, n, (const int *)L.rowptr, (const int *)L.slice_ptr, (const int *)L.scol,
+      launch_pdl(jac, g, TB, 0, st, n, sell_idx(s),
                  (const float *)L.sval32, (const float *)L.sinv32, (const float *)L.b32, xin, xout,
                  (const uint8_t *)L.skip);
       note_launches(1);
@@ -1781,10 +1774,9 @@ double time_smoother(System *s, int reps) {
   }
   if (!s->kz) fail(VAG_EINVAL, "no FP64 AMG hierarchy: solve with AMG first");
   auto sweep = [&](const double *xin, double *xout) {
-    auto jac = s->sell_u == 2 ? k_jac_sell<double, 2> : s->sell_u == 8 ? k_jac_sell<double, 8> : k_jac_sell<double, 4>;
-    launch_pdl(jac, g, TB, 0, st, n, (const int *)L.rowptr, (const int *)L.slice_ptr,
-               (const int *)L.scol, (const double *)L.sval, (const double *)L.sinv, (const double *)s->kr, xin, xout,
-               (const uint8_t *)L.skip);
+    auto jac = sell_pick(s, s->sell_u, [](auto u) { return k_jac_sell<double, decltype(u)::value>; });
+    launch_pdl(jac, g, TB, 0, st, n, sell_idx(s), (const double *)L.sval, (const double *)L.sinv,
+               (const double *)s->kr, xin, xout, (const uint8_t *)L.skip);
     note_launches(1);
   };
   VAG_CUDA(cudaMemsetAsync(s->kz, 0, sizeof(double) * n, st));

@@ -80,8 +80,7 @@ __global__ void __launch_bounds__(NT) k_jacobi_scale(const double *__restrict__ 
 // already done return at entry.  with_rz: also r.z and, in the last tile of
 // the system, beta = (r.z)' / (r.z), as k_rz does.
 template <int U>
-__global__ void __launch_bounds__(NT) k_cheb_step(const int *__restrict__ rowptr, const int *__restrict__ slice_ptr,
-                                                  const int *__restrict__ scol, const double *__restrict__ sval,
+__global__ void __launch_bounds__(NT) k_cheb_step(SellIdx ix, const double *__restrict__ sval,
                                                   const double *__restrict__ dinv, const double *__restrict__ r,
                                                   const double *__restrict__ coef, int j, const double *d_in,
                                                   const double *__restrict__ z_in, double *d_out,
@@ -100,7 +99,7 @@ __global__ void __launch_bounds__(NT) k_cheb_step(const int *__restrict__ rowptr
   if (valid) {
     const double ri = r[i];
     double di, zi;
-    cheb_row_step(c, j, ri, sell_row<double, U>(i, rowptr, slice_ptr, scol, sval, z_in), dinv[i], d_in[i], z_in[i],
+    cheb_row_step(c, j, ri, sell_row<double, U>(i, ix, sval, z_in), dinv[i], d_in[i], z_in[i],
                   &di, &zi);
     if (d_out) d_out[i] = di;
     z_out[i] = zi;
@@ -164,13 +163,13 @@ void cheb_apply(System *s, const double *r, double *z, cudaStream_t st, bool in_
     k_jacobi_scale<<<nt, NT, 0, st>>>(r, s->dinv, s->cw, tl);
     note_launches(1);
   }
-  auto step = s->sell_u == 2 ? k_cheb_step<2> : s->sell_u == 8 ? k_cheb_step<8> : k_cheb_step<4>;
+  auto step = sell_pick(s, s->sell_u, [](auto u) { return k_cheb_step<decltype(u)::value>; });
   const double *d_in = s->cw, *z_in = s->cw;
   for (int j = 1; j < kChebDegree; ++j) {
     const bool last = j == kChebDegree - 1;
     double *z_out = last ? z : (z_in == s->cy ? s->cw : s->cy);
     double *d_out = last ? nullptr : s->cd;
-    launch_pdl(step, nt, NT, 0, st, (const int *)s->rowptr, (const int *)s->slice_ptr, (const int *)s->scol,
+    launch_pdl(step, nt, NT, 0, st, sell_idx(s),
                (const double *)s->sval, (const double *)s->dinv, r, (const double *)s->cheb_coef, j, d_in, z_in,
                d_out, z_out, tl, s->partials, s->counter, s->ks, s->n_done, (int)in_iter, (int)(last && rz));
     note_launches(1);

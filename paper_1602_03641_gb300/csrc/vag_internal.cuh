@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <functional>
 #include <string>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -268,6 +269,8 @@ struct System {
   int sell_u = 0;              // loads in flight of the SELL row loop (0: not tuned yet)
   int *slice_ptr = nullptr;    // [n_slices+1] element offsets
   int *scol = nullptr;         // [sell_nnz]
+  unsigned short *scol16 = nullptr;   // [sell_nnz] and [n_slices], matrices that stream (SellIdx)
+  int *sbase = nullptr;
   double *sval = nullptr;      // [sell_nnz]
   double *rhs = nullptr;       // [n_rows]
   double *dinv = nullptr;      // [n_rows]
@@ -377,19 +380,76 @@ void sys_free_all(System *s);
 __device__ __forceinline__ float sell_val(__half v) { return __half2float(v); }
 __device__ __forceinline__ float sell_val(float v) { return v; }
 __device__ __forceinline__ double sell_val(double v) { return v; }
-template <class T, int U = 4, class V = T>
-__device__ __forceinline__ T sell_row(int row, const int *__restrict__ rowptr, const int *__restrict__ slice_ptr,
-                                      const int *__restrict__ scol, const V *__restrict__ sval,
-                                      const T *__restrict__ x) {
-  const int len = rowptr[row + 1] - rowptr[row];
-  const int base = slice_ptr[row >> 5] + (row & 31);
-  T s = 0;
+// A matrix that fits the L2 is read plainly.  A larger one streams through:
+// its entries pass L1 and L2 by with evict-first loads, so that the caches
+// keep x, and the columns are read as 16-bit offsets from the slice's smallest
+// column where the slice's columns span less than 2^16 (sbase >= 0; -1: as
+// they are).  On a lattice 32 consecutive rows reach two planes, so all but
+// the rows next to fractures qualify up to about 180 x 180 nodes a plane; an
+// entry then takes 10 instead of 12 bytes in FP64 and 6 instead of 8 in FP32.
+// At 128^3: FP64 product 138 -> 125 us, FP32 sweep 98 -> 83, FP32 product with
+// its sums 120 -> 102, mixed solve 38.1 -> 37.3 ms; at 80^3 the FP64 product
+// 30.5 -> 26.7.  (At 64^3, 84 MB, the streaming loads cost the FP32 sweep 9.4
+// -> 13.7 us, hence the rule; deciding inside one kernel instead of choosing
+// it cost a 64^3 run 0.6 %.  An explicit software pipeline over four entries
+// was 1.7 times slower in both.)
+constexpr size_t kStreamBytes = (size_t)128 << 20;   // FP64 values and columns; the L2 holds 129 MB
+struct SellIdx {
+  const int *rowptr, *slice_ptr, *scol;
+  const unsigned short *c16;   // [sell_nnz]
+  const int *sbase;            // [n_slices]
+};
+template <class T>
+__device__ __forceinline__ T ld_stream(const T *p) { return __ldcs(p); }
+__device__ __forceinline__ __half ld_stream(const __half *p) {
+  return __ushort_as_half(__ldcs(reinterpret_cast<const unsigned short *>(p)));
+}
+// s = f(s, value, column) over the entries of a row, in order; the loop is
+// unrolled |U| times, U < 0: the matrix streams
+template <int U, class T, class V, class F>
+__device__ __forceinline__ T sell_fold(int row, const SellIdx &ix, const V *__restrict__ sval, T s, F &&f) {
+  const int len = ix.rowptr[row + 1] - ix.rowptr[row];
+  const int base = ix.slice_ptr[row >> 5] + (row & 31);
+  if constexpr (U > 0) {
+    const int *__restrict__ c = ix.scol;
 #pragma unroll(U)
-  for (int k = 0; k < len; ++k) {
-    const int idx = base + 32 * k;
-    s = fma((T)sell_val(sval[idx]), x[scol[idx]], s);
+    for (int k = 0; k < len; ++k) {
+      const int p = base + 32 * k;
+      s = f(s, sval[p], c[p]);
+    }
+  } else {
+    const int cb = ix.sbase[row >> 5];
+    if (cb >= 0) {
+#pragma unroll(-U)
+      for (int k = 0; k < len; ++k) {
+        const int p = base + 32 * k;
+        s = f(s, ld_stream(sval + p), cb + (int)ld_stream(ix.c16 + p));
+      }
+    } else {
+#pragma unroll(-U)
+      for (int k = 0; k < len; ++k) {
+        const int p = base + 32 * k;
+        s = f(s, ld_stream(sval + p), ld_stream(ix.scol + p));
+      }
+    }
   }
   return s;
+}
+template <class T, int U = 4, class V = T>
+__device__ __forceinline__ T sell_row(int row, const SellIdx &ix, const V *__restrict__ sval,
+                                      const T *__restrict__ x) {
+  return sell_fold<U>(row, ix, sval, (T)0, [&](T s, V v, int j) { return fma((T)sell_val(v), x[j], s); });
+}
+
+inline SellIdx sell_idx(const System *s) { return {s->rowptr, s->slice_ptr, s->scol, s->scol16, s->sbase}; }
+// f(U) for an unroll of u (2, 4 or 8) of this system's matrix
+template <class F>
+auto sell_pick(const System *s, int u, F f) {
+  if (s->scol16)
+    return u == 2 ? f(std::integral_constant<int, -2>{}) : u == 8 ? f(std::integral_constant<int, -8>{})
+                                                                  : f(std::integral_constant<int, -4>{});
+  return u == 2 ? f(std::integral_constant<int, 2>{}) : u == 8 ? f(std::integral_constant<int, 8>{})
+                                                               : f(std::integral_constant<int, 4>{});
 }
 
 // ----------------------------------------------------------- utilities ----

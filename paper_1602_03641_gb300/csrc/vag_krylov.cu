@@ -32,8 +32,7 @@ constexpr int NT = 256;
 // q = A p in the sliced-ELL layout, one thread per row: exactly one FMA per
 // stored entry, in the row's CSR order.
 template <int U>
-__global__ void __launch_bounds__(NT) k_spmv(const int *__restrict__ rowptr, const int *__restrict__ slice_ptr,
-                                             const int *__restrict__ scol, const double *__restrict__ sval,
+__global__ void __launch_bounds__(NT) k_spmv(SellIdx ix, const double *__restrict__ sval,
                                              const double *__restrict__ x, double *__restrict__ y, Tiles tl,
                                              double *partials, unsigned *counter, KrylovScalars *ks, int *n_done,
                                              int with_dot) {
@@ -45,7 +44,7 @@ __global__ void __launch_bounds__(NT) k_spmv(const int *__restrict__ rowptr, con
   if (with_dot && ks[sys].done) return;
   double dp = 0.0;
   for (int row = r0 + threadIdx.x; row < r1; row += NT) {
-    const double s = sell_row<double, U>(row, rowptr, slice_ptr, scol, sval, x);
+    const double s = sell_row<double, U>(row, ix, sval, x);
     y[row] = s;
     dp = fma(x[row], s, dp);
   }
@@ -554,10 +553,9 @@ static void read_scalars(System *s) {
 }
 
 static void launch_spmv_u(System *s, int u, const double *x, double *y, int with_dot, cudaStream_t st) {
-  auto kern = u == 2 ? k_spmv<2> : u == 8 ? k_spmv<8> : k_spmv<4>;
-  launch_pdl(kern, s->seg.n_tiles, NT, 0, st, (const int *)s->rowptr, (const int *)s->slice_ptr,
-             (const int *)s->scol, (const double *)s->sval, x, y, tiles_of(s), s->partials, s->counter, s->ks,
-             s->n_done, with_dot);
+  auto kern = sell_pick(s, u, [](auto v) { return k_spmv<decltype(v)::value>; });
+  launch_pdl(kern, s->seg.n_tiles, NT, 0, st, sell_idx(s), (const double *)s->sval, x, y, tiles_of(s), s->partials,
+             s->counter, s->ks, s->n_done, with_dot);
   note_launches(1);
 }
 

@@ -52,8 +52,7 @@ __global__ void k_dscale(int n, const double *__restrict__ dinv, double *__restr
 }
 
 template <int U>
-__global__ void __launch_bounds__(NT) k_spmv32(const int *__restrict__ rowptr, const int *__restrict__ slice_ptr,
-                                               const int *__restrict__ scol, const float *__restrict__ sval,
+__global__ void __launch_bounds__(NT) k_spmv32(SellIdx ix, const float *__restrict__ sval,
                                                const float *__restrict__ x, float *__restrict__ y, Tiles tl,
                                                double *partials, unsigned *counter, KrylovScalars *ks, int *n_done) {
   const int t = blockIdx.x;
@@ -64,7 +63,7 @@ __global__ void __launch_bounds__(NT) k_spmv32(const int *__restrict__ rowptr, c
   const int r0 = tl.row0[t], r1 = tl.row1[t];
   float dp = 0.f;
   for (int row = r0 + threadIdx.x; row < r1; row += NT) {
-    const float s = sell_row<float, U>(row, rowptr, slice_ptr, scol, sval, x);
+    const float s = sell_row<float, U>(row, ix, sval, x);
     y[row] = s;
     dp = fmaf(x[row], s, dp);
   }
@@ -250,8 +249,7 @@ __global__ void k_dform_vals(int n, const int *__restrict__ rowptr, const int *_
 
 // q = A p in difference form and the partial p.q (as k_spmv32)
 template <int U>
-__global__ void __launch_bounds__(NT) k_spmv32d(const int *__restrict__ rowptr, const int *__restrict__ slice_ptr,
-                                                const int *__restrict__ scol, const float *__restrict__ sval,
+__global__ void __launch_bounds__(NT) k_spmv32d(SellIdx ix, const float *__restrict__ sval,
                                                 const float *__restrict__ rowsum, const float *__restrict__ x,
                                                 float *__restrict__ y, Tiles tl, double *partials, unsigned *counter,
                                                 KrylovScalars *ks, int *n_done) {
@@ -263,15 +261,9 @@ __global__ void __launch_bounds__(NT) k_spmv32d(const int *__restrict__ rowptr, 
   const int r0 = tl.row0[t], r1 = tl.row1[t];
   float dp = 0.f;
   for (int row = r0 + threadIdx.x; row < r1; row += NT) {
-    const int len = rowptr[row + 1] - rowptr[row];
-    const int base = slice_ptr[row >> 5] + (row & 31);
     const float pi = x[row];
-    float s = 0.f;
-#pragma unroll(U)
-    for (int k = 0; k < len; ++k) {   // the diagonal slot holds 0 and x_i - x_i = 0
-      const int idx = base + 32 * k;
-      s = fmaf(sval[idx], x[scol[idx]] - pi, s);
-    }
+    // the diagonal slot holds 0 and x_i - x_i = 0
+    float s = sell_fold<U>(row, ix, sval, 0.f, [&](float a, float v, int j) { return fmaf(v, x[j] - pi, a); });
     s = fmaf(rowsum[row], pi, s);
     y[row] = s;
     dp = fmaf(pi, s, dp);
@@ -467,7 +459,7 @@ static void ensure_mixed_buffers(System *s) {
 void mixed_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   ensure_krylov_buffers(s);
   tune_sell(s);
-  auto spmv32 = s->sell_u == 2 ? k_spmv32<2> : s->sell_u == 8 ? k_spmv32<8> : k_spmv32<4>;
+  auto spmv32 = sell_pick(s, s->sell_u, [](auto u) { return k_spmv32<decltype(u)::value>; });
   cudaStream_t st = s->ctx->stream;
   ensure_mixed_buffers(s);
   Mixed &m = s->mx;
@@ -488,7 +480,7 @@ void mixed_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   if (!m.loop.exec)
     loop_build(m.loop, st, [&](cudaGraphConditionalHandle h) {
       for (int i = 0; i < kLoopUnroll; ++i) {
-        spmv32<<<nt, NT, 0, st>>>(s->rowptr, s->slice_ptr, s->scol, m.sval32, m.p32, m.q32, tl, s->partials,
+        spmv32<<<nt, NT, 0, st>>>(sell_idx(s), m.sval32, m.p32, m.q32, tl, s->partials,
                                   s->counter, m.ks_in, m.n_done_in);
         k_upd32<<<nt, NT, 0, st>>>(m.x32, m.r32, m.p32, m.q32, tl, s->partials, s->counter, m.ks_in, m.n_done_in);
         k_pdir32<<<nt, NT, 0, st>>>(m.p32, m.r32, tl, m.ks_in, i + 1 == kLoopUnroll, h, m.n_done_in);
@@ -539,7 +531,7 @@ void mixed_amg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   trace_mark(st, "AMG setup (FP32 hierarchy), difference-form FP32 values");
   VAG_CUDA(cudaEventRecord(s->ev2, st));
   const float *a32 = m.dval32;   // FP32 difference-form values of A, sliced ELL
-  auto spmv32 = s->sell_u == 2 ? k_spmv32d<2> : s->sell_u == 8 ? k_spmv32d<8> : k_spmv32d<4>;
+  auto spmv32 = sell_pick(s, s->sell_u, [](auto u) { return k_spmv32d<decltype(u)::value>; });
   // one inner iteration, from r (and the V-cycle's first sweep) to the next r:
   // z = V(r) with r.z, p = z + beta p, q = A p with p.q, the update, which
   // forms the next first sweep and tests the inner tolerance (so that no
@@ -554,7 +546,7 @@ void mixed_amg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
       launch_pdl(k_irm_rz, nt, NT, 0, st, (const float *)m.r32, (const float *)m.z32, tl, s->partials, s->counter,
                  m.ks_in, m.n_done_in);
     launch_pdl(k_irm_pdir, nt, NT, 0, st, m.p32, (const float *)m.z32, tl, (const KrylovScalars *)m.ks_in);
-    launch_pdl(spmv32, nt, NT, 0, st, (const int *)s->rowptr, (const int *)s->slice_ptr, (const int *)s->scol, a32,
+    launch_pdl(spmv32, nt, NT, 0, st, sell_idx(s), a32,
                (const float *)m.rowsum32, (const float *)m.p32, m.q32, tl, s->partials, s->counter, m.ks_in,
                m.n_done_in);
     launch_pdl(k_irm_update, nt, NT, 0, st, m.x32, m.r32, (const float *)m.p32, (const float *)m.q32, tl, s->partials,
@@ -598,12 +590,12 @@ double time_spmv32(System *s, int reps) {
   Mixed &m = s->mx;
   const int n = s->n_rows, ns = s->seg.n_sys, nt = s->seg.n_tiles;
   const Tiles tl = tiles_of(s);
-  auto spmv32 = s->sell_u == 2 ? k_spmv32d<2> : s->sell_u == 8 ? k_spmv32d<8> : k_spmv32d<4>;
+  auto spmv32 = sell_pick(s, s->sell_u, [](auto u) { return k_spmv32d<decltype(u)::value>; });
   k_fill32<<<grid_for(n, NT), NT, 0, st>>>(n, 1.0f, m.p32);
   note_launches(1);
   VAG_CUDA(cudaMemsetAsync(m.ks_in, 0, sizeof(KrylovScalars) * ns, st));   // done = 0 everywhere
   auto launch = [&]() {
-    launch_pdl(spmv32, nt, NT, 0, st, (const int *)s->rowptr, (const int *)s->slice_ptr, (const int *)s->scol,
+    launch_pdl(spmv32, nt, NT, 0, st, sell_idx(s),
                (const float *)m.dval32, (const float *)m.rowsum32, (const float *)m.p32, m.q32, tl, s->partials,
                s->counter, m.ks_in, m.n_done_in);
     note_launches(1);

@@ -5,6 +5,8 @@
 // (no cross-lane reduction -- on GB300 the FP64 pipe, not HBM, limits a
 // lane-split CSR SpMV).  Entries of a row keep their CSR order, so a row sum
 // is the same sequence of FMAs whatever the slice layout.
+#include <climits>
+
 #include "vag_internal.cuh"
 
 namespace vag {
@@ -40,6 +42,31 @@ __global__ void k_sell_pad(int n, const int *__restrict__ rowptr, const int *__r
   const int len = row < n ? rowptr[row + 1] - rowptr[row] : 0;
   const int base = slice_ptr[sl] + (row & 31);
   for (int k = len; k < w; ++k) scol[base + 32 * k] = row < n ? row : 0;
+}
+
+// One warp per slice: the slice's smallest column and the 16-bit offsets from
+// it, or -1 where they do not fit (the columns then stay 32-bit).
+__global__ void __launch_bounds__(TB) k_sell_pack(int n, int n_slices, const int *__restrict__ slice_ptr,
+                                                  const int *__restrict__ scol, unsigned short *__restrict__ c16,
+                                                  int *__restrict__ sbase) {
+  const int sl = blockIdx.x * (TB / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (sl >= n_slices) return;   // whole warps
+  const int b = slice_ptr[sl], e = slice_ptr[sl + 1];
+  const bool mine = sl * 32 + lane < n;   // past the last row the columns are 0
+  int lo = INT_MAX, hi = -1;
+  for (int p = b + lane; p < e; p += 32) {
+    const int c = scol[p];
+    if (mine) {
+      lo = min(lo, c);
+      hi = max(hi, c);
+    }
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  const bool fits = hi >= 0 && hi - lo < 65536;
+  if (lane == 0) sbase[sl] = fits ? lo : -1;
+  if (!fits) return;
+  for (int p = b + lane; p < e; p += 32) c16[p] = mine ? (unsigned short)(scol[p] - lo) : (unsigned short)0;
 }
 
 template <class T>
@@ -89,6 +116,14 @@ void build_sell(System *s, int64_t total) {
     k_sell_cols<<<grid_for(n, TB), TB, 0, st>>>(n, s->rowptr, s->col, s->slice_ptr, s->scol);
     k_sell_pad<<<grid_for((int64_t)s->n_slices * 32, TB), TB, 0, st>>>(n, s->rowptr, s->slice_ptr, s->scol);
     note_launches(2);
+    // (a context with a budget keeps to the arrays that the budget was set for)
+    if ((size_t)total * 12 > kStreamBytes && !s->ctx->budget) {
+      s->scol16 = sys_alloc<unsigned short>(s, (size_t)total);
+      s->sbase = sys_alloc<int>(s, (size_t)s->n_slices);
+      k_sell_pack<<<grid_for(s->n_slices, TB / 32), TB, 0, st>>>(n, s->n_slices, s->slice_ptr, s->scol, s->scol16,
+                                                                 s->sbase);
+      note_launches(1);
+    }
     VAG_CHECK_LAUNCH();
   }
 }
