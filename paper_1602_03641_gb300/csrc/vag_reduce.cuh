@@ -65,68 +65,156 @@ struct Tiles {
   int n_tiles, n_sys;
 };
 
-// Sums K values per system in two levels, so that no counter sees more than
-// about kSegGroup or n_tiles / kSegGroup arrivals (a system of 8 000 tiles
-// otherwise queues 8 000 atomics on one address): per-tile block sums go to
-// partials[K*t + k]; the last tile of a group to arrive adds the group's
-// tile partials in tile order into partials[K*(n_tiles + g) + k]; the last
-// group of system `sys` to finish adds its group partials in group order and
-// returns true in all its threads with out[] valid in thread 0.  The grouping
-// depends on the system alone, so the sums do too.  Counters: counter[sys]
-// per system, counter[n_sys + 1 + g] per group.
+// Counts this thread in; true for the last of `members`, which then also sees
+// what the others wrote before they counted.  (A __threadfence() on every
+// member would also acquire, that is, drop the SM's L1 lines under the tiles
+// that still gather from it.)
+__device__ __forceinline__ bool arrive_last(unsigned *counter, int members) {
+  unsigned t;
+  asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(counter) : "memory");
+  if (t != (unsigned)(members - 1)) return false;
+  asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  return true;
+}
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// out[k] = the sum of ng group partials, as a block would form it: thread b
+// adds the groups b, b + NT, ..., then the warps' sums are added.  One warp;
+// load(k, b) gives a group's partial.
+template <int NT, int K, class F>
+__device__ __forceinline__ void groups_sum(int ng, int lane, double (&out)[K], F &&load) {
+  constexpr int NW = NT / 32;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    double acc[NW];
+#pragma unroll
+    for (int w = 0; w < NW; ++w) acc[w] = w * 32 + lane < ng ? load(k, w * 32 + lane) : 0.0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w)
+      for (int b = w * 32 + lane + NT; b < ng; b += NT) acc[w] += load(k, b);
+    double mine = 0.0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+      if (w * 32 >= ng) break;
+      const double sw = warp_sum(acc[w]);
+      if (lane == w) mine = sw;
+    }
+    out[k] = warp_sum(mine);
+  }
+}
+
+// Sums K values per system: per-tile block sums go to partials[K*t + k]; the
+// tiles of a group of kSegGroup are added in tile order, then the groups in
+// group order.  True in thread 0 of one tile alone, where out[] holds the
+// sums.  The grouping depends on the system alone, so the sums do too (also
+// on which of the two ways below they are taken).
+// Every Krylov kernel of a small system waits for this chain and little else
+// (a barrier, a write, a fence, an atomic and a read of the L2 a level, about
+// 3 us), so it is kept short.  A system of one tile needs no counter; up to
+// one group, its last tile's first warp adds the partials alone.  Up to
+// kSegOneLevel tiles the last tile of the system to arrive (counter[sys])
+// adds everything, a group a warp: one releasing atomic and one read of the
+// partials.  A larger system would queue thousands of atomics on one address:
+// the last tile of each group (counter[n_sys + 1 + g]) writes the group's sum
+// to partials[K*(n_tiles + g) + k], and the last of those groups adds them.
+// Against two levels for all, with a __threadfence() and barriers in each:
+// 8^3 cells with Jacobi CG (3 tiles) 4.54 -> 3.68 ms, 29 x 23 x 19 cells (51
+// tiles) 7.34 -> 6.88, 48^3 mixed solve (457 tiles) 12.50 -> 11.74, 64^3 run
+// (1060 tiles) 24.37 -> 23.89, 128^3 run (8637 tiles) 130.8 ms in both.
+// (Two levels with one warp each instead of the block for 33 to 1024 tiles:
+// 7.19 and 12.61 ms; the block for the 3 tiles: 3.90 ms.)
+// One call a kernel (the shared words are not guarded against a second).
+constexpr int kSegOneLevel = 1024;
 template <int NT, int K>
 __device__ __forceinline__ bool seg_sum(const double (&v)[K], double *partials, unsigned *counter, const Tiles &tl,
                                         int t, int sys, double (&out)[K]) {
-  __shared__ double sh[NT / 32];
+  static_assert(kSegGroup == 32, "a group's tiles are one warp's lanes");
+  constexpr int NW = NT / 32;
+  __shared__ double sh[K][NW];
+  __shared__ double gsum[K][kSegOneLevel / kSegGroup];
   __shared__ bool last;
-  double bs[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) bs[k] = block_sum<NT>(v[k], sh);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int t0 = tl.sys_tile0[sys], t1 = tl.sys_tile0[sys + 1];
+  const int ng = (t1 - t0 + kSegGroup - 1) / kSegGroup;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const double w = warp_sum(v[k]);
+    if (lane == 0) sh[k][warp] = w;
+  }
+  __syncthreads();
+  if (t1 - t0 > kSegGroup && t1 - t0 <= kSegOneLevel) {
+    if (warp == 0) {
+#pragma unroll
+      for (int k = 0; k < K; ++k) out[k] = warp_sum(lane < NW ? sh[k][lane] : 0.0);
+    }
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int k = 0; k < K; ++k) partials[(size_t)K * t + k] = out[k];
+      last = arrive_last(&counter[sys], t1 - t0);
+    }
+    __syncthreads();
+    if (!last) return false;
+    // a warp's groups, all loads first
+    constexpr int kMine = kSegOneLevel / kSegGroup / NW;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      double g[kMine];
+#pragma unroll
+      for (int q = 0; q < kMine; ++q) {
+        const int b = t0 + (q * NW + warp) * kSegGroup + lane;
+        g[q] = b < t1 ? __ldcg(&partials[(size_t)K * b + k]) : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < kMine; ++q) {
+        if (q * NW + warp >= ng) break;
+        const double sg = warp_sum(g[q]);
+        if (lane == 0) gsum[k][q * NW + warp] = sg;
+      }
+    }
+    __syncthreads();
+    if (warp != 0) return false;
+    groups_sum<NT, K>(ng, lane, out, [&](int k, int b) { return gsum[k][b]; });
+    if (lane == 0) counter[sys] = 0u;
+    return lane == 0;
+  }
+  if (warp != 0) return false;
+#pragma unroll
+  for (int k = 0; k < K; ++k) out[k] = warp_sum(lane < NW ? sh[k][lane] : 0.0);
+  const int grp = tl.grp0[sys];
   const int gl = (t - t0) / kSegGroup;                 // group within the system
   const int ga = t0 + gl * kSegGroup;                  // its tiles [ga, gb)
   const int gb = min(ga + kSegGroup, t1);
-  const int g = tl.grp0[sys] + gl;                     // its storage index
-  const int ng = tl.grp0[sys + 1] - tl.grp0[sys];
-  unsigned *gctr = counter + tl.n_sys + 1;
+  const int g = grp + gl;                              // its storage index
+  if (t1 - t0 == 1) return lane == 0;
+  unsigned *gctr = ng == 1 ? counter + sys : counter + tl.n_sys + 1 + g;
   double *gpart = partials + (size_t)K * tl.n_tiles;
-  if (threadIdx.x == 0) {
+  bool mine = false;
+  if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < K; ++k) partials[(size_t)K * t + k] = bs[k];
-    __threadfence();
-    const unsigned ticket = atomicAdd(&gctr[g], 1u);
-    last = (ticket == (unsigned)(gb - ga - 1));
+    for (int k = 0; k < K; ++k) partials[(size_t)K * t + k] = out[k];
+    mine = arrive_last(gctr, gb - ga);
   }
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-  double gs[K];
+  if (!__shfl_sync(0xffffffffu, mine, 0)) return false;
+  __syncwarp();
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    double acc = 0.0;
-    for (int b = ga + threadIdx.x; b < gb; b += NT) acc += __ldcg(&partials[(size_t)K * b + k]);
-    gs[k] = block_sum<NT>(acc, sh);
-  }
-  if (threadIdx.x == 0) {
-    gctr[g] = 0u;
+  for (int k = 0; k < K; ++k)
+    out[k] = warp_sum(ga + lane < gb ? __ldcg(&partials[(size_t)K * (ga + lane) + k]) : 0.0);
+  if (lane == 0) *gctr = 0u;
+  if (ng == 1) return lane == 0;
+  if (lane == 0) {
 #pragma unroll
-    for (int k = 0; k < K; ++k) gpart[(size_t)K * g + k] = gs[k];
-    __threadfence();
-    const unsigned ticket = atomicAdd(&counter[sys], 1u);
-    last = (ticket == (unsigned)(ng - 1));
+    for (int k = 0; k < K; ++k) gpart[(size_t)K * g + k] = out[k];
+    mine = arrive_last(&counter[sys], ng);
   }
-  __syncthreads();
-  if (!last) return false;
-  __threadfence();
-  const int g0 = tl.grp0[sys];
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < ng; b += NT) acc += __ldcg(&gpart[(size_t)K * (g0 + b) + k]);
-    out[k] = block_sum<NT>(acc, sh);
-  }
-  if (threadIdx.x == 0) counter[sys] = 0u;
-  return true;
+  if (!__shfl_sync(0xffffffffu, mine, 0)) return false;
+  __syncwarp();
+  groups_sum<NT, K>(ng, lane, out, [&](int k, int b) { return __ldcg(&gpart[(size_t)K * (grp + b) + k]); });
+  if (lane == 0) counter[sys] = 0u;
+  return lane == 0;
 }
 
 }  // namespace vag
