@@ -82,6 +82,36 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// The sum of a 256-thread tile's values sh[thread], valid in all lanes of the
+// calling warp: the tree of warp_sum in every warp, then over the warps'
+// sums, on the same pairs, but each partial sum formed once instead of in
+// every lane that could use it: 12 FP64 instructions a tile instead of 45.
+// (The FP64 pipe takes about 16 cycles an SM for a warp instruction, so the
+// 45 were 700 cycles a tile, more than the loads of a short FP32 kernel.
+// 64^3 run 23.55 -> 23.1 ms, 96^3 solve 31.9 -> 31.5, 128^3 run 129.9 -> 129.4;
+// the FP32 update with its sum in the 128^3 solve 60.5 -> 47.1 us.)
+__device__ __forceinline__ double tile_sum(const double *sh, int lane) {
+  double a[4];   // lanes l and l + 16 of warps 2 j + (lane >> 4), l = lane & 15
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const double *p = sh + (2 * j + (lane >> 4)) * 32 + (lane & 15);
+    a[j] = p[0] + p[16];
+  }
+  const bool h8 = lane & 8, h4 = lane & 4;   // these bits pick j from here on
+  double b0 = h8 ? a[2] : a[0], b1 = h8 ? a[3] : a[1];
+  b0 += __shfl_xor_sync(0xffffffffu, h8 ? a[0] : a[2], 8);
+  b1 += __shfl_xor_sync(0xffffffffu, h8 ? a[1] : a[3], 8);
+  double c = h4 ? b1 : b0;
+  c += __shfl_xor_sync(0xffffffffu, h4 ? b0 : b1, 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+  // the warps: bits 2, 1, 0 of their number are lane bits 3, 2, 4
+  c += __shfl_xor_sync(0xffffffffu, c, 8);
+  c += __shfl_xor_sync(0xffffffffu, c, 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 16);
+  return c;
+}
+
 // out[k] = the sum of ng group partials, as a block would form it: thread b
 // adds the groups b, b + NT, ..., then the warps' sums are added.  One warp;
 // load(k, b) gives a group's partial.
@@ -134,22 +164,20 @@ __device__ __forceinline__ bool seg_sum(const double (&v)[K], double *partials, 
                                         int t, int sys, double (&out)[K]) {
   static_assert(kSegGroup == 32, "a group's tiles are one warp's lanes");
   constexpr int NW = NT / 32;
-  __shared__ double sh[K][NW];
+  static_assert(NT == 256, "tile_sum");
+  __shared__ double sh[K][NT];
   __shared__ double gsum[K][kSegOneLevel / kSegGroup];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int t0 = tl.sys_tile0[sys], t1 = tl.sys_tile0[sys + 1];
   const int ng = (t1 - t0 + kSegGroup - 1) / kSegGroup;
 #pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const double w = warp_sum(v[k]);
-    if (lane == 0) sh[k][warp] = w;
-  }
+  for (int k = 0; k < K; ++k) sh[k][threadIdx.x] = v[k];
   __syncthreads();
   if (t1 - t0 > kSegGroup && t1 - t0 <= kSegOneLevel) {
     if (warp == 0) {
 #pragma unroll
-      for (int k = 0; k < K; ++k) out[k] = warp_sum(lane < NW ? sh[k][lane] : 0.0);
+      for (int k = 0; k < K; ++k) out[k] = tile_sum(sh[k], lane);
     }
     if (threadIdx.x == 0) {
 #pragma unroll
@@ -183,7 +211,7 @@ __device__ __forceinline__ bool seg_sum(const double (&v)[K], double *partials, 
   }
   if (warp != 0) return false;
 #pragma unroll
-  for (int k = 0; k < K; ++k) out[k] = warp_sum(lane < NW ? sh[k][lane] : 0.0);
+  for (int k = 0; k < K; ++k) out[k] = tile_sum(sh[k], lane);
   const int grp = tl.grp0[sys];
   const int gl = (t - t0) / kSegGroup;                 // group within the system
   const int ga = t0 + gl * kSegGroup;                  // its tiles [ga, gb)
