@@ -428,25 +428,41 @@ __global__ void k_cv_sys(int nv, int nf, int nc, int n_sys, const int *__restric
 // widest row (rows of a slice have nearly equal counts, see k_sigma_sort).
 // Launched with programmatic dependent launch: the map (written once per
 // solve) is read before the dependency wait, the previous step's c after it.
-// The map streams through once a step (evict-first loads), so the cache keeps
-// the concentrations that the gathers reuse.
+// A map larger than the L2 streams through once a step (evict-first loads), so
+// that the cache keeps the concentrations that the gathers reuse.  Where the
+// map and the state (12 bytes a stored entry, three doubles a row) take at
+// most kStepFits, the map is read plainly and stays: us a step with
+// evict-first and with plain loads at 36^3 x 6 tetrahedra (21 MB) 9.3 / 8.1,
+// 64^3 (39 MB) 8.25 / 7.75, 72^3 11.1 / 10.2, 80^3 (75 MB) 14.8 / 13.6, but
+// 88^3 (102 MB) 18.4 / 19.4, 140 x 90 x 61 (115 MB) 19.7 / 22.7 and 128^3
+// (317 MB) 49.7 / 58.5.  (L1::no_allocate loads were slower than both in all of
+// them; 16-bit column offsets gave 128^3 48.4, 140 x 90 x 61 19.6 and smaller
+// maps nothing, about what packing them costs; five or six entries ahead of
+// the wait instead of four are 10 and 20 % slower on hexahedra.)
 constexpr int kStepPF = 4;
 constexpr int kStepTB = 128;   // 128 / 256 / 512 threads: 54.8 / 55.3 / 58.7 us at 128^3
+constexpr size_t kStepFits = (size_t)80 << 20;
+template <bool FITS, class T>
+__device__ __forceinline__ T ld_map(const T *p) {
+  if constexpr (FITS) return __ldg(p);
+  else return __ldcs(p);
+}
+template <bool FITS>
 __global__ void __launch_bounds__(kStepTB) k_step(int n, const int *__restrict__ sp, const int *__restrict__ col,
                                                   const double *__restrict__ w, const double *__restrict__ diag,
                                                   const double *__restrict__ c, double *__restrict__ cn) {
   const int i = blockIdx.x * kStepTB + threadIdx.x;
   if ((i >> 5) >= (n + 31) >> 5) return;   // whole warps
   const int r = i & 31;
-  const int k0 = __ldcs(sp + (i >> 5)), width = (__ldcs(sp + (i >> 5) + 1) - k0) >> 5;
+  const int k0 = ld_map<FITS>(sp + (i >> 5)), width = (ld_map<FITS>(sp + (i >> 5) + 1) - k0) >> 5;
   const bool valid = i < n;
-  const double d = valid ? __ldcs(diag + i) : 0.0;
+  const double d = valid ? ld_map<FITS>(diag + i) : 0.0;
   int pc[kStepPF];
   double pw[kStepPF];
 #pragma unroll
   for (int u = 0; u < kStepPF; ++u) {
-    pc[u] = valid && u < width ? __ldcs(col + k0 + 32 * u + r) : 0;
-    pw[u] = valid && u < width ? __ldcs(w + k0 + 32 * u + r) : 0.0;
+    pc[u] = valid && u < width ? ld_map<FITS>(col + k0 + 32 * u + r) : 0;
+    pw[u] = valid && u < width ? ld_map<FITS>(w + k0 + 32 * u + r) : 0.0;
   }
   pdl_wait();
   pdl_trigger();
@@ -455,7 +471,7 @@ __global__ void __launch_bounds__(kStepTB) k_step(int n, const int *__restrict__
 #pragma unroll
   for (int u = 0; u < kStepPF; ++u)
     if (u < width) v = fma(pw[u], c[pc[u]], v);
-  for (int u = kStepPF; u < width; ++u) v = fma(__ldcs(w + k0 + 32 * u + r), c[__ldcs(col + k0 + 32 * u + r)], v);
+  for (int u = kStepPF; u < width; ++u) v = fma(ld_map<FITS>(w + k0 + 32 * u + r), c[ld_map<FITS>(col + k0 + 32 * u + r)], v);
   cn[i] = v;
 }
 
@@ -478,6 +494,11 @@ __global__ void k_set_dir(int nd, const int *__restrict__ dn, const double *__re
   if (i < nd) c[dn[i]] = cbar[i];
 }
 
+// entries of 12 bytes, and three vectors
+auto step_kernel(const System *s) {
+  return 12 * (size_t)s->t_cap + 24 * (size_t)s->t_rows <= kStepFits ? k_step<true> : k_step<false>;
+}
+
 }  // namespace
 
 // Mean duration of one explicit step on the current upwind map.
@@ -488,7 +509,7 @@ double time_transport_step(System *s, int reps) {
   const int gs = grid_for(32 * ((n + 31) / 32), kStepTB);
   double *a = s->cbuf, *b = s->cbuf + n;
   auto step = [&](const double *c, double *cn) {
-    launch_pdl(k_step, gs, kStepTB, 0, st, n, (const int *)s->tsp, (const int *)s->tcol, (const double *)s->tval,
+    launch_pdl(step_kernel(s), gs, kStepTB, 0, st, n, (const int *)s->tsp, (const int *)s->tcol, (const double *)s->tval,
                (const double *)s->tdiag, c, cn);
     note_launches(1);
   };
@@ -626,7 +647,7 @@ void transport_run(System *s, const vag_transport_opts *o, double *c_dev, vag_tr
       set_capturing(true);
       double *a = s->cbuf, *b = s->cbuf + nt;
       for (int k = 0; k < kStepChunk; ++k) {
-        launch_pdl(k_step, gs, kStepTB, 0, st, nt, (const int *)s->tsp, (const int *)s->tcol, (const double *)s->tval,
+        launch_pdl(step_kernel(s), gs, kStepTB, 0, st, nt, (const int *)s->tsp, (const int *)s->tcol, (const double *)s->tval,
                    (const double *)s->tdiag, (const double *)a, b);
         std::swap(a, b);
       }
@@ -643,7 +664,7 @@ void transport_run(System *s, const vag_transport_opts *o, double *c_dev, vag_tr
     }
   }
   for (int k = chunks * kStepChunk; k < o->n_steps; ++k) {
-    launch_pdl(k_step, gs, kStepTB, 0, st, nt, (const int *)s->tsp, (const int *)s->tcol, (const double *)s->tval,
+    launch_pdl(step_kernel(s), gs, kStepTB, 0, st, nt, (const int *)s->tsp, (const int *)s->tcol, (const double *)s->tval,
                (const double *)s->tdiag, (const double *)c0, c1);
     note_launches(1);
     std::swap(c0, c1);
