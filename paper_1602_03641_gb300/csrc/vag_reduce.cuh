@@ -156,7 +156,9 @@ __device__ __forceinline__ void groups_sum(int ng, int lane, double (&out)[K], F
 // tiles) 7.34 -> 6.88, 48^3 mixed solve (457 tiles) 12.50 -> 11.74, 64^3 run
 // (1060 tiles) 24.37 -> 23.89, 128^3 run (8637 tiles) 130.8 ms in both.
 // (Two levels with one warp each instead of the block for 33 to 1024 tiles:
-// 7.19 and 12.61 ms; the block for the 3 tiles: 3.90 ms.)
+// 7.19 and 12.61 ms; the block for the 3 tiles: 3.90 ms.  One level up to 2048 or
+// 4096 tiles: 64^3 run 0.5 and 2 % slower, 96^3 solve, 3733 tiles, the same
+// and 3 % slower.)
 // One call a kernel (the shared words are not guarded against a second).
 constexpr int kSegOneLevel = 1024;
 template <int NT, int K>
