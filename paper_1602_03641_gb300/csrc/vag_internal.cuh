@@ -320,8 +320,7 @@ struct System {
   int64_t t_cap = 0;
   double *cbuf = nullptr;      // [2 (n_cv + n_perf)]
   double *dts = nullptr;       // [2 n_sys]: per system dt_max, dt
-  cudaGraphExec_t step_graph = nullptr;   // kStepChunk transport steps
-  int64_t step_graph_cap = -1;
+  cudaGraphExec_t step_graph = nullptr;   // kStepChunk transport steps over the arrays above
   int step_graph_rows = 0;
   int t_rows = 0;              // rows allocated for tdiag, tperm, tsp and each half of cbuf
   std::vector<double> dts_host;

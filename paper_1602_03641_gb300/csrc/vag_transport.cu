@@ -573,7 +573,14 @@ void transport_run(System *s, const vag_transport_opts *o, double *c_dev, vag_tr
     note_launches(1);
   }
   const int n_slices = (nt + 31) / 32;
+  // the kept graph of steps holds the addresses of the arrays that grow below,
+  // and the kernel that their sizes choose
+  auto drop_steps = [&] {
+    if (s->step_graph) cudaGraphExecDestroy(s->step_graph);
+    s->step_graph = nullptr;
+  };
   if (nt > s->t_rows) {
+    drop_steps();
     s->tdiag = sys_alloc<double>(s, nt);
     s->tperm = sys_alloc<int>(s, nt);
     s->tsp = sys_alloc<int>(s, (size_t)n_slices + 1);
@@ -612,6 +619,7 @@ void transport_run(System *s, const vag_transport_opts *o, double *c_dev, vag_tr
   if (n_stored < (int64_t)nnz_t) fail(VAG_EINVAL, "the transport map exceeds 2^31 stored entries");
   if (n_stored > s->t_cap) {
     // grow the entry arrays (kept across calls)
+    drop_steps();
     s->tcol = sys_alloc<int>(s, (size_t)std::max<int64_t>(n_stored, 1));
     s->tval = sys_alloc<double>(s, (size_t)std::max<int64_t>(n_stored, 1));
     s->t_cap = n_stored;
@@ -639,9 +647,8 @@ void transport_run(System *s, const vag_transport_opts *o, double *c_dev, vag_tr
   constexpr int kStepChunk = 20;
   const int chunks = o->n_steps / kStepChunk;
   if (chunks > 0) {
-    if (!s->step_graph || s->step_graph_cap != s->t_cap || s->step_graph_rows != nt) {
-      if (s->step_graph) cudaGraphExecDestroy(s->step_graph);
-      s->step_graph = nullptr;
+    if (!s->step_graph || s->step_graph_rows != nt) {
+      drop_steps();
       cudaGraph_t graph;
       VAG_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
       set_capturing(true);
@@ -655,7 +662,6 @@ void transport_run(System *s, const vag_transport_opts *o, double *c_dev, vag_tr
       VAG_CUDA(cudaStreamEndCapture(st, &graph));
       VAG_CUDA(cudaGraphInstantiate(&s->step_graph, graph, 0));
       cudaGraphDestroy(graph);
-      s->step_graph_cap = s->t_cap;
       s->step_graph_rows = nt;
     }
     for (int c = 0; c < chunks; ++c) {
