@@ -1235,7 +1235,7 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
   A.levels.push_back(L0);
   int *undecided = static_cast<int *>(alloc(sizeof(int)));
   int *pin = ctx_pin(s->ctx);
-  int *dense_status = s->status + 1;   // set by the inversions of the terminal blocks, read once at the end
+  int *dense_status = s->status + 1;   // set by the inversions of the terminal blocks, read by amg_check_status
   VAG_CUDA(cudaMemsetAsync(dense_status, 0, sizeof(int), st));
   for (int lvl = 0;; ++lvl) {
     if (lvl == kMaxLevels) fail(VAG_ECUDA, "AMG: hierarchy deeper than the level cap");
@@ -1430,7 +1430,6 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
     if (!A.levels.empty()) A.levels[0].r32 = static_cast<float *>(alloc(4 * (size_t)std::max(A.levels[0].n, 1)));
   }
   VAG_CUDA(cudaMemcpyAsync(&pin[kDenseStatusPin], dense_status, sizeof(int), cudaMemcpyDeviceToHost, st));
-  A.status_pending = true;   // checked when the caller waits for the solve
   // first nonzero of each system on every coarse level (the tail's layout)
   const bool may_tail = f32 && !classical;   // the one-kernel tail walks aggregates
   for (size_t l = 1; may_tail && l < A.levels.size(); ++l) {
@@ -1497,10 +1496,11 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
 }
 
 void amg_check_status(System *s) {
-  if (!s->amg.status_pending) return;
-  s->amg.status_pending = false;
-  if (ctx_pin(s->ctx)[kDenseStatusPin] & ST_NONPOSITIVE)
+  VAG_CUDA(cudaStreamSynchronize(s->ctx->stream));
+  if (ctx_pin(s->ctx)[kDenseStatusPin] & ST_NONPOSITIVE) {
+    s->amg.built = false;
     fail(VAG_EINVAL, "AMG: a terminal block is not positive definite");
+  }
 }
 
 // Level arrays of one precision.

@@ -367,7 +367,14 @@ void gmres_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   // the Arnoldi steps of a cycle, kChunk to a graph (rebuilt every solve:
   // the preconditioner's buffers are new each time)
   const int nchunks = (kRestart + kChunk - 1) / kChunk;
-  std::vector<cudaGraphExec_t> chunks(nchunks, nullptr);
+  struct Chunks {   // released on every path
+    std::vector<cudaGraphExec_t> g;
+    ~Chunks() {
+      for (cudaGraphExec_t e : g)
+        if (e) cudaGraphExecDestroy(e);
+    }
+  } built{std::vector<cudaGraphExec_t>(nchunks, nullptr)};
+  std::vector<cudaGraphExec_t> &chunks = built.g;
   std::vector<size_t> chunk_nodes(nchunks, 0);
   for (int c = 0; c < nchunks; ++c) {
     cudaGraph_t graph;
@@ -380,6 +387,7 @@ void gmres_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     VAG_CUDA(cudaGraphInstantiate(&chunks[c], graph, 0));
     cudaGraphDestroy(graph);
   }
+  if (amg) amg_check_status(s);
   VAG_CUDA(cudaMemsetAsync(s->kx, 0, sizeof(double) * s->n_rows, st));
   restart(1);
   int *pin = ctx_pin(s->ctx);
@@ -405,8 +413,6 @@ void gmres_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     note_launches(1);
     restart(0);
   }
-  for (auto &g : chunks)
-    if (g) cudaGraphExecDestroy(g);
   // the true residual decides the status
   true_residual2(s, st);
   finish_solve(s, info, false);

@@ -141,7 +141,6 @@ struct Amg {
   std::vector<void *> allocs;
   size_t bytes = 0;
   bool built = false;
-  bool status_pending = false;     // the terminal blocks' status is on its way to the pinned words
   bool f32 = false;                // V-cycle in FP32
   bool classical = false;          // classical (Ruge-Stueben-type) levels instead of aggregation
   int tail_start = -1;             // first level run by the one-kernel tail
@@ -565,7 +564,9 @@ bool amg_apply_cg(System *s, const double *r, double *z, cudaStream_t st);
 const float *amg_first_sweep_scale_f32(System *s, float *&t0, float &omega);
 bool amg_apply_f32_cg(System *s, const float *r, float *z, cudaStream_t st, KrylovScalars *ks, int *n_done);
 void amg_free(System *s);
-// after a wait for the stream: fails if a terminal block of the last setup was not positive definite
+// Waits for the setup; fails if one of its terminal blocks was not positive
+// definite.  Every solve calls it before its first V-cycle, and so before any
+// result is written: its host work (the capture of the loop) lies between.
 void amg_check_status(System *s);
 // Chebyshev preconditioner (FP64): cheb_setup estimates each system's interval
 // from Jacobi-CG Lanczos coefficients and fills the coefficient table;

@@ -797,6 +797,7 @@ void pcg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     });
     trace_mark(st, "loop capture + instantiate");
   }
+  if (amg) amg_check_status(s);
   // The recursive residual can drift below the true one; after convergence
   // the true residual is recomputed and CG restarts from the current iterate
   // (a few times at most) for every system still above its tolerance whose
@@ -896,6 +897,7 @@ void bicgstab_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
     k_bi_pdir<<<nt, NT, 0, st>>>(s->kp, s->kr, s->kq, tl, s->ks, h, s->n_done);
     note_launches(5);
   });
+  if (amg) amg_check_status(s);
   VAG_CUDA(cudaGraphLaunch(s->bicg_loop.exec, st));
   note_loop(s, s->bicg_loop);
   // the true residual decides the status
@@ -935,7 +937,6 @@ void finish_solve(System *s, vag_solve_info *info, bool mixed) {
   trace_mark(st, "scatter + cell recovery + fluxes");
   VAG_CUDA(cudaEventRecord(s->ev1, st));
   read_scalars(s);
-  amg_check_status(s);
   float ms = 0.f;
   cudaEventElapsedTime(&ms, s->ev0, s->ev1);
   // aggregate over the batch: most iterations, worst residual, worst status

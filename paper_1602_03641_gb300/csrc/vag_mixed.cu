@@ -560,6 +560,7 @@ void mixed_amg_solve(System *s, const vag_solve_opts *o, vag_solve_info *info) {
   // the hierarchy is rebuilt every solve, so is the loop of inner iterations
   loop_build(m.loop_amg, st, iteration);
   trace_mark(st, "loop capture + instantiate");
+  amg_check_status(s);
   const double eta_min = o->inner_rtol > 0.0 ? o->inner_rtol : kEtaAmg;
   for (int outer = 0; outer < kMaxOuter + 1; ++outer) {
     if (poll(s, outer, m.loop_amg)) break;
