@@ -1188,12 +1188,9 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
   const int ns = s->seg.n_sys;
   // the device memory of a previous hierarchy is reused only if the
   // structure matches; simplest: free the old one (its allocations are
-  // tracked separately from the system's)
-  for (void *p : A.allocs) ctx_free(s->ctx, p);
-  A.allocs.clear();
-  A.levels.clear();
-  s->ctx->in_use -= A.bytes;
-  A.bytes = 0;
+  // tracked separately from the system's).  No hierarchy until this one is
+  // complete: a setup that fails half way leaves none.
+  amg_free(s);
   // small arrays share chunks: a hierarchy has a few hundred, most of a few KB
   unsigned char *chunk = nullptr;
   size_t chunk_left = 0;

@@ -69,3 +69,19 @@ def test_indefinite_terminal_block(ctx, precision, precond, krylov, zero_rhs):
     s.solve(rtol=1e-12)
     solve()
     s.close()
+
+
+# 251 unknowns, whose coarse operators have non-positive diagonals (FP64 and FP32 hierarchies): the setup ends
+# before its levels are complete
+@pytest.mark.parametrize("precision", [vag.VAG_FP64, vag.VAG_MIXED])
+@pytest.mark.parametrize("precond", [vag.VAG_PC_AMG, vag.VAG_PC_AMG_RS])
+def test_a_setup_that_fails_half_way_leaves_no_hierarchy(ctx, precision, precond):
+    pb = vi.random_dfn_problem(6, 1, 1e2, 5)
+    s = vag.assemble_problem(ctx, pb)
+    s.solve(precision=precision, precond=precond, rtol=1e-10)
+    assert s.kernel_time(vag.VAG_KERNEL_SMOOTH, 1) > 0.0
+    bad = np.tile([1.0, 1.0, 1.0, 2.0, 0.0, 0.0], pb.n_cells)
+    s.update_props(bad, pb.lambda_f, pb.d_f, pb.mu)
+    refused(lambda: s.solve(precision=precision, precond=precond, rtol=1e-10, maxit=50))
+    refused(lambda: s.kernel_time(vag.VAG_KERNEL_SMOOTH, 1))
+    s.close()
