@@ -1192,13 +1192,14 @@ void amg_setup(System *s, bool f32, bool f16, bool classical) {
   // complete: a setup that fails half way leaves none.
   amg_free(s);
   // small arrays share chunks: a hierarchy has a few hundred, most of a few KB
+  // (not under a budget, which counts what each array takes)
   unsigned char *chunk = nullptr;
   size_t chunk_left = 0;
   std::function<void *(size_t)> alloc = [&](size_t bytes) -> void * {
     constexpr size_t kSmall = 32 << 10, kChunk = 256 << 10;
     bytes = (bytes + 255) & ~size_t(255);
     if (!bytes) bytes = 256;
-    if (bytes <= kSmall) {
+    if (bytes <= kSmall && !s->ctx->budget) {
       if (bytes > chunk_left) {
         chunk = static_cast<unsigned char *>(alloc(kChunk));
         chunk_left = kChunk;
