@@ -199,7 +199,13 @@ typedef struct {
 
 /* Create a context on CUDA device `device`.  mem_budget_bytes caps the device
  * memory all systems of this context may hold (0 = no cap).  The context owns
- * a non-blocking stream unless vag_ctx_set_stream() supplies one. */
+ * a non-blocking stream unless vag_ctx_set_stream() supplies one, and a pool:
+ * device memory of destroyed systems and of the calls' own scratch stays in it
+ * for reuse until the context is freed.  The scratch counts neither in the cap
+ * nor in vag_ctx_bytes_in_use().  Without a cap a matrix of more than 128 MiB
+ * (12 bytes a stored entry) also holds its columns as 16-bit offsets, 2 bytes
+ * an entry more, which its products read faster; with one it holds none.  The
+ * results are the same. */
 vag_status vag_ctx_create(int device, size_t mem_budget_bytes, vag_ctx **out);
 /* Release the context.  Systems created from it stay valid; the context's
  * resources are freed with the last of them.  No new system may be created

@@ -154,7 +154,6 @@ struct Amg {
   double *s0d = nullptr;
 };
 
-// State of the mixed-precision solve (FP32 inner CG inside FP64 refinement).
 // A loop that the device ends: a CUDA graph whose single node repeats its
 // body while its condition is non-zero (it starts at 1 with every launch; a
 // kernel of the body sets it to 0, see loop_end_check).  Against graphs of 8
@@ -168,6 +167,7 @@ struct LoopGraph {
   size_t nodes = 0;              // kernels of one pass over the body
 };
 
+// State of the mixed-precision solve (FP32 inner CG inside FP64 refinement).
 struct Mixed {
   float *sval32 = nullptr;     // FP32 sliced-ELL values of S A S, S = D^{-1/2} (Jacobi)
   float *x32 = nullptr, *r32 = nullptr, *p32 = nullptr, *q32 = nullptr;
@@ -338,7 +338,8 @@ void ctx_free(Ctx *c, void *p);
 constexpr int kPinWords = 64;
 int *ctx_pin(Ctx *c);
 // Pinned staging buffer of at least `bytes` bytes.  Callers wait for the
-// stream before they read it and before they ask for it again.
+// stream before the host reads it, writes it again or asks for more bytes;
+// copies to and from it follow one another on the context's stream.
 void *ctx_stage(Ctx *c, size_t bytes);
 // Temporaries of the context's pool, stream-ordered, released on every path.
 // (The device's default pool hands its memory back to the driver at every
@@ -378,19 +379,28 @@ void sys_free_all(System *s);
 __device__ __forceinline__ float sell_val(__half v) { return __half2float(v); }
 __device__ __forceinline__ float sell_val(float v) { return v; }
 __device__ __forceinline__ double sell_val(double v) { return v; }
-// A matrix that fits the L2 is read plainly.  A larger one streams through:
-// its entries pass L1 and L2 by with evict-first loads, so that the caches
-// keep x, and the columns are read as 16-bit offsets from the slice's smallest
-// column where the slice's columns span less than 2^16 (sbase >= 0; -1: as
-// they are).  On a lattice 32 consecutive rows reach two planes, so all but
-// the rows next to fractures qualify up to about 180 x 180 nodes a plane; an
-// entry then takes 10 instead of 12 bytes in FP64 and 6 instead of 8 in FP32.
-// At 128^3: FP64 product 138 -> 125 us, FP32 sweep 98 -> 83, FP32 product with
-// its sums 120 -> 102, mixed solve 38.1 -> 37.3 ms; at 80^3 the FP64 product
-// 30.5 -> 26.7.  (At 64^3, 84 MB, the streaming loads cost the FP32 sweep 9.4
-// -> 13.7 us, hence the rule; deciding inside one kernel instead of choosing
-// it cost a 64^3 run 0.6 %.  An explicit software pipeline over four entries
-// was 1.7 times slower in both.)
+// A matrix whose FP64 values and columns take at most kStreamBytes (about the
+// L2's 129 MB) is read plainly.  A larger one streams through: its entries
+// pass L1 and L2 by with evict-first loads, so that the caches keep x, and the
+// columns are read as 16-bit offsets from the slice's smallest column where
+// the slice's columns span less than 2^16 (sbase >= 0; -1: as they are).  On a
+// lattice 32 consecutive rows reach two planes, so all but the rows next to
+// fractures qualify up to about 180 x 180 nodes a plane; an entry then takes
+// 10 instead of 12 bytes in FP64, 6 instead of 8 in FP32, 4 instead of 6 in
+// FP16.  The FP32 and FP16 copies follow the same line although they are
+// smaller: inside a solve they share the L2 with the rest of the hierarchy.
+// Plain / streamed (us; mixed aggregation and FP16 solves in ms), fractured
+// lattices of n cells a side:
+//   n (FP64 MB)   FP64 product   FP32 sweep    FP32 product   mixed solve   FP16 solve
+//   74 (132)      36.8 / 32.3    21.4 / 22.3   28.3 / 30.1    15.6 / 13.8   15.4 / 14.0
+//   80 (166)      39.3 / 35.0    27.5 / 23.2   36.4 / 32.6    17.0 / 15.0   17.5 / 15.7
+//   96 (287)      59.3 / 52.5    42.5 / 34.4   53.1 / 45.4    27.2 / 25.0   27.8 / 26.2
+//   112 (456)     91.4 / 80.3    64.9 / 51.5   80.5 / 66.4    48.9 / 45.4   46.7 / 44.3
+// (the sweep and the product alone, launched again and again, keep the FP32
+// copy of 74 cells a side, 88 MB, in the L2).  At 64 cells a side, 84 MB, the
+// streaming loads cost the FP32 sweep 9.4 -> 13.7 us, hence the rule; deciding
+// inside one kernel instead of choosing it cost a run there 0.6 %.  An
+// explicit software pipeline over four entries was 1.7 times slower in both.
 constexpr size_t kStreamBytes = (size_t)128 << 20;   // FP64 values and columns; the L2 holds 129 MB
 struct SellIdx {
   const int *rowptr, *slice_ptr, *scol;

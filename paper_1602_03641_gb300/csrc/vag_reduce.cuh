@@ -152,7 +152,7 @@ __device__ __forceinline__ void groups_sum(int ng, int lane, double (&out)[K], F
 // the last tile of each group (counter[n_sys + 1 + g]) writes the group's sum
 // to partials[K*(n_tiles + g) + k], and the last of those groups adds them.
 // Against two levels for all, with a __threadfence() and barriers in each:
-// 8^3 cells with Jacobi CG (3 tiles) 4.54 -> 3.68 ms, 29 x 23 x 19 cells (51
+// 8^3 cells with Jacobi CG (3 tiles) 4.53 -> 3.64 ms, 29 x 23 x 19 cells (51
 // tiles) 7.34 -> 6.88, 48^3 mixed solve (457 tiles) 12.50 -> 11.74, 64^3 run
 // (1060 tiles) 24.37 -> 23.89, 128^3 run (8637 tiles) 130.8 ms in both.
 // (Two levels with one warp each instead of the block for 33 to 1024 tiles:
